@@ -227,7 +227,9 @@ lbm_status lbm_step(lbm_grid_t g, int64_t n_coarse_steps);
  * max_variants)) (nullable) the measured time per coarse step of each (the
  * longer timing for the two fastest), n_variants (nullable) their number.
  * Synchronises the bound stream; drops captured step graphs.  Without a call
- * the grid uses variant 0.  The paper has no counterpart. */
+ * the grid uses the variant a rule on its tiles and size gives (isothermal:
+ * kernel 1 or the 64-node tiles, samples beside the pass on small grids;
+ * thermal: variant 0).  The paper has no counterpart. */
 lbm_status lbm_autotune(lbm_grid_t g, int32_t trials, int32_t* chosen, float* ms_per_step, int32_t max_variants,
                         int32_t* n_variants);
 

@@ -546,6 +546,33 @@ lbm_status run_instant(lbm_grid* g, int k) {
   return LBM_OK;
 }
 
+// The variant a grid runs until lbm_autotune or lbm_set_variant chooses one.
+// Kernel 1 (128-node tiles, two load stages, 4 CTAs per SM) is the faster or
+// within 1% of the fastest on rows that fill its tiles: 3.23 ms a step against
+// kernel 0's 3.55 on the 256 x 64 x 128 channel, 2.02 against 2.25 on the
+// sphere.  The 64-node tiles take over where they leave a quarter of the lanes
+// fewer idle: 24^3 box 8.2 us against 9.9, 32^3 FP64 two-level box 0.260 ms
+// against 0.275 (kernel 0: 0.444), 27 x 53 x 108 BF16 box 0.067 against 0.079;
+// at equal lanes they lose (20 x 49 x 25 FP64 channel 2.40 against 2.00).  The
+// samples run beside the pass below a million node updates an instant, where
+// the pass leaves the GPU idle (64^3 two-level box, 0.39 M: 0.086 ms against
+// 0.093; reduced curved sphere, 0.5 M: 0.447 against 0.461); the sphere at
+// 4.3 M loses 6% by it.  The thermal model keeps its kernel 0.
+void default_variant(lbm_grid* g) {
+  if (g->hg.thermal) return;
+  double l128 = 0, l64 = 0, updates = 0;
+  for (const auto& p : g->hg.P) {
+    const double n = (double)(1LL << p.level);
+    for (int k = 0; k < 2; ++k) {
+      l128 += n * 128.0 * (double)p.tiles_pure[k].size();
+      l64 += n * 64.0 * (double)p.tiles_half[k].size();
+    }
+    updates += n * (double)p.n_fluid;
+  }
+  g->variant = l64 <= 0.75 * l128 ? lbmk::sc_tma_variants(g->hg.desc.storage) - 1 : 1;
+  g->presample = updates < 1e6 * (double)(1LL << (g->hg.nlev - 1));
+}
+
 }  // namespace
 
 extern "C" {
@@ -603,6 +630,7 @@ lbm_status lbm_grid_create(const lbm_desc* desc, lbm_grid_t* out) {
     off += (b + 255) / 256 * 256;
     return o;
   };
+  default_variant(g);
   g->off_status = take(64);
   g->off_partial = take(sizeof(double) * 8 * kDiagBlocks * hg.P.size());
   g->off_diag_out = take(sizeof(double) * 8);
