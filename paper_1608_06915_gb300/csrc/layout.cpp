@@ -522,10 +522,14 @@ std::string build_layout(HostGrid& g) {
                 if (act[k]) odd_nodes[k].push_back((uint32_t)m);
           }
           const uint32_t id = (uint32_t)((z * p.dim[1] + y) * p.ntx + tx);
-          // the TMA path fetches the periodic wrap of x-spanning rows as 16-byte
-          // boxes at x = dim - H: row-edge tiles need dim a multiple of 8 nodes
+          // the TMA path fetches the periodic wrap of x-spanning rows as aligned
+          // 16-byte boxes, so rows of any length can take it (a row of one node
+          // would need both wraps at once).  FP64 thermal rows of odd lengths
+          // stay on the node-by-node kernel: that collision is bound by the FP64
+          // pipe, and the tile pass keeps fewer warps on it.
           const bool edge = tx == 0 || (tx + 1) * 128 >= p.dim[0];
-          const bool wrap_ok = !p.span[0] || !edge || p.dim[0] % 8 == 0;
+          const bool wrap_ok = !p.span[0] || !edge || p.dim[0] % 8 == 0 ||
+                               (p.dim[0] >= 2 && !(g.thermal && g.pop_bytes == 8));
           for (int k = 0; k < 2; ++k) {
             if (active[k] == 0) continue;
             R.all[k].push_back(id);

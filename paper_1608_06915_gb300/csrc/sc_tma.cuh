@@ -244,6 +244,13 @@ __device__ __forceinline__ constexpr int row_base(int i) {
 // their tile lists; each tile carries its patch's tensor maps, geometry,
 // relaxation and force.
 constexpr int kTmaBatch = 8;  // patches per launch
+
+// The 16-byte wrap box of a row's last node: its first element and the last
+// node's place in it.
+template <int H>
+__device__ __forceinline__ int wrap_box_x(int dim) { return (dim - 1) & ~(H - 1); }
+template <int H>
+__device__ __forceinline__ int wrap_box_at(int dim) { return (dim - 1) & (H - 1); }
 constexpr long long kWarpNodes = 152 * 4 * 128;  // fix-up lists up to this size go one warp per node
 
 template <typename S, typename R>
@@ -338,7 +345,7 @@ __global__ void __launch_bounds__(BX + 32, MINB) k_sc_tma(const __grid_constant_
             continue;
           }
           tma_load_row(stage + j * C::GROUP, &E.map_in, &full[s], x0, sy, sz, 3 * j);
-          if (first) tma_load_row(side + j * C::SIDE, &E.map_wrap, &full[s], p.dim[0] - C::H, sy, sz, 3 * j + 2);
+          if (first) tma_load_row(side + j * C::SIDE, &E.map_wrap, &full[s], wrap_box_x<C::H>(p.dim[0]), sy, sz, 3 * j + 2);
           if (last) tma_load_row(side + (9 + j) * C::SIDE, &E.map_wrap, &full[s], 0, sy, sz, 3 * j);
         }
       }
@@ -382,10 +389,11 @@ __global__ void __launch_bounds__(BX + 32, MINB) k_sc_tma(const __grid_constant_
       // periodic wrap along x from the side slots (rows not bounced)
       const S* side = reinterpret_cast<const S*>(smem + s * C::STAGE + 9 * C::GROUP);
       const bool lo = x == 0;
+      const int at = wrap_box_at<C::H>(p.dim[0]);
       unroll<27>([&](auto I) {
         constexpr int i = decltype(I)::value;
         const bool b = (bm >> (i / 3)) & 1;
-        if (!b && lo && CX(i) == 1) f[i] = SCvt<S>::to(side[(i / 3) * (C::SIDE / (int)sizeof(S)) + C::H - 1]);
+        if (!b && lo && CX(i) == 1) f[i] = SCvt<S>::to(side[(i / 3) * (C::SIDE / (int)sizeof(S)) + at]);
         if (!b && !lo && CX(i) == -1) f[i] = SCvt<S>::to(side[(9 + i / 3) * (C::SIDE / (int)sizeof(S))]);
       });
     }
@@ -499,7 +507,7 @@ __device__ __forceinline__ void issue_tile(const TmaBatch<S, float>& b, int t, u
     const int sy = wrap_axis(ty - (j % 3 - 1), p.dim[1]);
     const int sz = wrap_axis(tz - (j / 3 - 1), p.dim[2]);
     tma_load_row(stage + j * C::GROUP, &E.map_in, full, x0, sy, sz, 3 * j);
-    if (first) tma_load_row(side + j * C::SIDE, &E.map_wrap, full, p.dim[0] - C::H, sy, sz, 3 * j + 2);
+    if (first) tma_load_row(side + j * C::SIDE, &E.map_wrap, full, wrap_box_x<C::H>(p.dim[0]), sy, sz, 3 * j + 2);
     if (last) tma_load_row(side + (9 + j) * C::SIDE, &E.map_wrap, full, 0, sy, sz, 3 * j);
   }
 }
@@ -573,11 +581,12 @@ __global__ void __launch_bounds__(NP * 64, MINB) k_sc_tma2(const __grid_constant
     const bool lo_edge = xa == 0, hi_a = xa == p.dim[0] - 1, hi_b = xa + 1 == p.dim[0] - 1;
     if (p.span[0] && (lo_edge || hi_a || hi_b)) {
       const S* side = reinterpret_cast<const S*>(smem + s * C::STAGE + 9 * C::GROUP);
+      const int at = wrap_box_at<C::H>(p.dim[0]);
       unroll<27>([&](auto I) {
         constexpr int i = decltype(I)::value;
         if ((bm >> (i / 3)) & 1) return;
         if constexpr (CX(i) == 1) {
-          if (lo_edge) f[i].v.x = SCvt<S>::to(side[(i / 3) * (C::SIDE / (int)sizeof(S)) + C::H - 1]);
+          if (lo_edge) f[i].v.x = SCvt<S>::to(side[(i / 3) * (C::SIDE / (int)sizeof(S)) + at]);
         }
         if constexpr (CX(i) == -1) {
           const float w = SCvt<S>::to(side[(9 + i / 3) * (C::SIDE / (int)sizeof(S))]);

@@ -105,7 +105,7 @@ __device__ __forceinline__ void th_tma_body(const ThMaps<R>& m, const PatchDev& 
           const int sy = wrap_axis(ty - (j % 3 - 1), p.dim[1]);
           const int sz = wrap_axis(tz - (j / 3 - 1), p.dim[2]);
           tma_load_row(half + j * C::GROUP, in, &full[s], x0, sy, sz, 3 * j);
-          if (first) tma_load_row(side + j * C::SIDE, wr, &full[s], p.dim[0] - C::H, sy, sz, 3 * j + 2);
+          if (first) tma_load_row(side + j * C::SIDE, wr, &full[s], wrap_box_x<C::H>(p.dim[0]), sy, sz, 3 * j + 2);
           if (last) tma_load_row(side + (9 + j) * C::SIDE, wr, &full[s], 0, sy, sz, 3 * j);
         }
       }
@@ -169,12 +169,13 @@ __device__ __forceinline__ void th_tma_body(const ThMaps<R>& m, const PatchDev& 
       const R* sf = stf + 9 * C::GROUP / (int)sizeof(R);
       const R* sg = stg + 9 * C::GROUP / (int)sizeof(R);
       const bool lo = x == 0;
+      const int at = wrap_box_at<C::H>(p.dim[0]);
       unroll<27>([&](auto I) {
         constexpr int i = decltype(I)::value;
         const bool b = (bm >> (i / 3)) & 1;
         if (!b && lo && CX(i) == 1) {
-          f[i] = sf[(i / 3) * (C::SIDE / (int)sizeof(R)) + C::H - 1];
-          g[i] = sg[(i / 3) * (C::SIDE / (int)sizeof(R)) + C::H - 1];
+          f[i] = sf[(i / 3) * (C::SIDE / (int)sizeof(R)) + at];
+          g[i] = sg[(i / 3) * (C::SIDE / (int)sizeof(R)) + at];
         }
         if (!b && !lo && CX(i) == -1) {
           f[i] = sf[(9 + i / 3) * (C::SIDE / (int)sizeof(R))];
