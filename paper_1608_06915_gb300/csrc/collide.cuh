@@ -232,6 +232,72 @@ __host__ __device__ constexpr int shear_class() {
   return 0;
 }
 
+// Tables of the product-form equilibrium in deviation form.  With the per-axis
+// deviations d and 1 + q_xy = (1 + d_x)(1 + d_y),
+//   f^eq_i - W_i = W_i (rho~ + rho q_i) = W1(c_z) (B + d_z A),
+//   A = W_xy rho (1 + q_xy),  B = W_xy (rho~ + rho q_xy),
+// each a product or a sum of same-sized deviations (no cancellation).  W1 is
+// 1/6 at +-1 and 4/6 at 0, so with the 1/6 of every axis in the tables only a
+// factor 4 is left at c = 0: a column (c_x, c_y) costs one multiply, one or
+// two FMAs and an FMA per layer, against a table of q_xy and three operations
+// a population.  The collision is bound by instruction issue (70% of the slots
+// at FP32, more with 16-bit storage) and at FP64 by the FP64 pipe, so its
+// operation count is its time: k_sc_tma's operations on a node fell by about
+// 100 of 640 (32^3 two-level box at FP64: 4.78 to 4.50 ms per ten steps; the
+// channel at FP32: 3.44 to 3.37 ms a step).
+template <typename V>
+struct EqTables {
+  V ax[3], bx[3], bx4[3];  // per c_x: A and B of the axis, each with W1(c_x)/36; 4 B
+  V dy[3], gy[3];          // per c_y: 6 W1(c_y) times d_y and 1 + d_y
+  __device__ __forceinline__ EqTables(V rho_t, V rho, const V (&dx)[3], const V (&dyv)[3]) {
+    const V one = K<V>(1.0), four = K<V>(4.0);
+    const V r1 = K<V>(1.0 / 216.0) * rho, t1 = K<V>(1.0 / 216.0) * rho_t;
+    const V r4 = four * r1, t4 = four * t1;
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+      const V r = c == 1 ? r4 : r1, t = c == 1 ? t4 : t1;
+      ax[c] = vfma(r, dx[c], r);
+      bx[c] = vfma(r, dx[c], t);
+      bx4[c] = four * bx[c];
+      dy[c] = c == 1 ? four * dyv[c] : dyv[c];
+      gy[c] = (c == 1 ? four : one) + dy[c];
+    }
+  }
+  // A and B of column (a, b), the 1/6 of the z axis included: f^eq - W is
+  // B + d_z A at c_z = +-1, 4 (B + d_z A) at 0
+  __device__ __forceinline__ void column(int a, int b, V& A, V& B) const {
+    A = ax[a] * gy[b];
+    B = vfma(dy[b], ax[a], b == 1 ? bx4[a] : bx[a]);
+  }
+};
+
+// The same from a table of q_xy and the four weight classes, in the order of
+// operations of the 16-bit storages: there a last bit of FP32 moves the
+// rounding of the stored value, so EqTables, no less exact, gives velocities
+// that differ by 3e-4 (FP16) and 2e-3 (BF16) after four steps of the channel,
+// the storage's own error.  They keep this order (EqTables: 3.8% faster).
+template <typename V>
+struct EqClasses {
+  V wr[4], wrt[4], qxy[3][3];
+  __device__ __forceinline__ EqClasses(V rho_t, V rho, const V (&dx)[3], const V (&dy)[3]) {
+    constexpr double WK[4] = {8.0 / 27.0, 2.0 / 27.0, 1.0 / 54.0, 1.0 / 216.0};
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      wr[k] = K<V>(WK[k]) * rho;
+      wrt[k] = K<V>(WK[k]) * rho_t;
+    }
+#pragma unroll
+    for (int a = 0; a < 3; ++a)
+#pragma unroll
+      for (int b = 0; b < 3; ++b) qxy[a][b] = vfma(dx[a], dy[b], dx[a] + dy[b]);
+  }
+  template <int i>
+  __device__ __forceinline__ V dev(const V (&dzs)[3]) const {
+    const V t = qxy[CX(i) + 1][CY(i) + 1], dz = dzs[CZ(i) + 1];
+    return vfma(wr[wclass<i>()], vfma(t, dz, t + dz), wrt[wclass<i>()]);
+  }
+};
+
 // The collision of Eqs. f_equations, f_mirr, gamma_min_approx in delta form,
 //   f'_i = f^eq_i + (1 - beta gamma) df_i + beta (gamma - 2) ds_i,
 // df = f - f^eq, ds the shear part (reading: natural-moment basis), with the
@@ -241,41 +307,42 @@ __host__ __device__ constexpr int shear_class() {
 // by the post-collision deviations; returns gamma.  With DF, f holds df itself
 // on entry (a state assembled as f^eq(rho, u) + df, whose df is known).  FM:
 // compile-time mask of the axes along which du may be nonzero (0: no force).
+// TAB: f^eq from EqTables (FP32 and FP64 storage) or EqClasses (16-bit).
 // beta and du are the same for every node of V (a pair of nodes shares its
 // patch).
 //
 // Every per-direction quantity is a product of per-axis factors, so the loops
-// read small tables: q_i from (1 + q_xy)(1 + d_z) - 1, rho W_i from the four
-// weight classes, the second moments from the three z-columns of each
-// (c_x, c_y) pair, the entropic weights 1/f^eq_i as 1/(g_x g_y) per column
+// read small tables: f^eq from EqTables, the second moments from the three
+// z-columns of each (c_x, c_y) pair, the entropic weights 1/f^eq_i as 1/(g_x g_y) per column
 // times 1/(rho g_z) per layer.  The tables of f^eq are built twice (before
 // and after gamma) rather than held, which keeps few values live.
-template <typename V, int FM, bool DF = false>
+template <typename V, int FM, bool DF = false, bool TAB = true>
 __device__ __forceinline__ V kbc_collide_v(V (&f)[27], V rho_t, V rho, V ux, V uy, V uz, V beta, V dux, V duy,
                                            V duz, bool du_x, bool du_y, bool du_z, bool lbgk) {
   AxisV<V> ex, ey, ez;
   axis_eq_v<V>(ux, ex, !lbgk);
   axis_eq_v<V>(uy, ey, !lbgk);
   axis_eq_v<V>(uz, ez, !lbgk);
-  // f^eq_i - W_i = W_i (rho~ + rho q_i), q_i = (1 + q_xy)(1 + d_z) - 1, from
-  // the per-axis deviations; f becomes df = f - f^eq
-  constexpr double WK[4] = {8.0 / 27.0, 2.0 / 27.0, 1.0 / 54.0, 1.0 / 216.0};
-  if constexpr (!DF) {
-    V wr[4], wrt[4], qxy[3][3];
-#pragma unroll
-    for (int k = 0; k < 4; ++k) {
-      wr[k] = K<V>(WK[k]) * rho;
-      wrt[k] = K<V>(WK[k]) * rho_t;
-    }
-#pragma unroll
-    for (int a = 0; a < 3; ++a)
-#pragma unroll
-      for (int b = 0; b < 3; ++b) qxy[a][b] = vfma(ex.d[a], ey.d[b], ex.d[a] + ey.d[b]);
+  // f becomes df = f - f^eq
+  if constexpr (!DF && !TAB) {
+    const EqClasses<V> T(rho_t, rho, ex.d, ey.d);
     unroll<27>([&](auto I) {
       constexpr int i = decltype(I)::value;
-      const V t = qxy[CX(i) + 1][CY(i) + 1], dz = ez.d[CZ(i) + 1];
-      f[i] = f[i] - vfma(wr[wclass<i>()], vfma(t, dz, t + dz), wrt[wclass<i>()]);
+      f[i] = f[i] - T.template dev<i>(ez.d);
     });
+  } else if constexpr (!DF) {
+    const EqTables<V> T(rho_t, rho, ex.d, ey.d);
+#pragma unroll
+    for (int b = 0; b < 3; ++b)
+#pragma unroll
+      for (int c = 0; c < 3; ++c) {
+        V A, B;
+        T.column(c, b, A, B);
+        const int j = c + 3 * b;
+        f[j] = f[j] - vfma(ez.d[0], A, B);
+        f[j + 18] = f[j + 18] - vfma(ez.d[2], A, B);
+        f[j + 9] = vfma(K<V>(-4.0), vfma(ez.d[1], A, B), f[j + 9]);
+      }
   }
   // second moments of df: per (c_x, c_y) column, z0 = sum over c_z,
   // z1 = sum c_z df, z2 = sum c_z^2 df
@@ -377,23 +444,27 @@ __device__ __forceinline__ V kbc_collide_v(V (&f)[27], V rho_t, V rho, V ux, V u
       for (int c = 0; c < 3; ++c) dzz[c] = sh.d[c];
     }
   }
-  V wr[4], wrt[4], qxy[3][3];
-#pragma unroll
-  for (int k = 0; k < 4; ++k) {
-    wr[k] = K<V>(WK[k]) * rho;
-    wrt[k] = K<V>(WK[k]) * rho_t;
+  if constexpr (!TAB) {
+    const EqClasses<V> T(rho_t, rho, dx, dy);
+    unroll<27>([&](auto I) {
+      constexpr int i = decltype(I)::value, sc = shear_class<i>();
+      const V e = T.template dev<i>(dzz);
+      if constexpr (sc == 0) f[i] = vfma(a, f[i], e);
+      else f[i] = vfma(a, f[i], e + bds[sc]);
+    });
+    return gamma;
   }
-#pragma unroll
-  for (int ca = 0; ca < 3; ++ca)
-#pragma unroll
-    for (int cb = 0; cb < 3; ++cb) qxy[ca][cb] = vfma(dx[ca], dy[cb], dx[ca] + dy[cb]);
-  unroll<27>([&](auto I) {
-    constexpr int i = decltype(I)::value;
-    constexpr int sc = shear_class<i>();
-    const V t = qxy[CX(i) + 1][CY(i) + 1], dz = dzz[CZ(i) + 1];
-    const V e = vfma(wr[wclass<i>()], vfma(t, dz, t + dz), wrt[wclass<i>()]);
-    if constexpr (sc == 0) f[i] = vfma(a, f[i], e);
-    else f[i] = vfma(a, f[i], e + bds[sc]);
+  const EqTables<V> T(rho_t, rho, dx, dy);
+  unroll<9>([&](auto J) {
+    constexpr int j = decltype(J)::value;
+    V A, B;
+    T.column(j % 3, j / 3, A, B);
+    unroll<3>([&](auto C) {
+      constexpr int c = decltype(C)::value, i = j + 9 * c, sc = shear_class<i>();
+      const V e = vfma(dzz[c], A, B);  // f^eq - W; a quarter of it at c_z = 0
+      if constexpr (sc == 0) f[i] = vfma(a, f[i], c == 1 ? K<V>(4.0) * e : e);
+      else f[i] = vfma(a, f[i], c == 1 ? vfma(K<V>(4.0), e, bds[sc]) : e + bds[sc]);
+    });
   });
   return gamma;
 }
@@ -409,14 +480,15 @@ struct CollideType<float> {
   using V = F1;
 };
 
-// DF: f holds df = f - f^eq(rho, u) on entry (kbc_collide_v).
-template <typename R, int FM, bool DF = false>
+// DF: f holds df = f - f^eq(rho, u) on entry (kbc_collide_v).  S: the storage
+// type of the populations.
+template <typename R, int FM, bool DF = false, typename S = R>
 __device__ __forceinline__ R kbc_collide_m(R (&f)[27], R rho_t, R rho, R ux, R uy, R uz, R beta, R dux, R duy,
                                            R duz, bool lbgk) {
   using V = typename CollideType<R>::V;
   V fv[27];
   unroll<27>([&](auto I) { fv[decltype(I)::value] = V(f[decltype(I)::value]); });
-  const V g = kbc_collide_v<V, FM, DF>(fv, V(rho_t), V(rho), V(ux), V(uy), V(uz), V(beta), V(dux), V(duy),
+  const V g = kbc_collide_v<V, FM, DF, (sizeof(S) > 2)>(fv, V(rho_t), V(rho), V(ux), V(uy), V(uz), V(beta), V(dux), V(duy),
                                        V(duz), dux != R(0), duy != R(0), duz != R(0), lbgk);
   unroll<27>([&](auto I) {
     constexpr int i = decltype(I)::value;
@@ -427,14 +499,14 @@ __device__ __forceinline__ R kbc_collide_m(R (&f)[27], R rho_t, R rho, R ux, R u
   else return g.v;
 }
 
-template <typename R, int FM>
+template <typename R, int FM, typename S = R>
 __device__ __forceinline__ R kbc_collide(R (&f)[27], R beta, R dux, R duy, R duz, bool lbgk) {
   using V = typename CollideType<R>::V;
   V fv[27];
   unroll<27>([&](auto I) { fv[decltype(I)::value] = V(f[decltype(I)::value]); });
   V rho_t, rho, ux, uy, uz;
   macro_v<V>(fv, rho_t, rho, ux, uy, uz);
-  const V g = kbc_collide_v<V, FM>(fv, rho_t, rho, ux, uy, uz, V(beta), V(dux), V(duy), V(duz), dux != R(0),
+  const V g = kbc_collide_v<V, FM, false, (sizeof(S) > 2)>(fv, rho_t, rho, ux, uy, uz, V(beta), V(dux), V(duy), V(duz), dux != R(0),
                                    duy != R(0), duz != R(0), lbgk);
   unroll<27>([&](auto I) {
     constexpr int i = decltype(I)::value;

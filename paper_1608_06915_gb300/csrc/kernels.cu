@@ -81,7 +81,7 @@ __global__ void __launch_bounds__(128) k_coalesce(PatchDev pc, const S* __restri
     constexpr int i = decltype(I)::value;
     f[i] = fe[i] + rescale * (f[i] - fe[i]);
   });
-  kbc_collide<R, FM>(f, beta_p, dux, duy, duz, lbgk != 0);
+  kbc_collide<R, FM, S>(f, beta_p, dux, duy, duz, lbgk != 0);
   store_node<S, R>(pp, fout_p, cf_parent[k], f);
 }
 
@@ -244,7 +244,7 @@ __device__ __forceinline__ void explode_node(const PatchDev& pc, S* __restrict__
       f[i] = ip(4 + i);
     });
   }
-  kbc_collide_m<R, FM, true>(f, m[0], R(1) + m[0], m[1], m[2], m[3], beta_c, dux, duy, duz, lbgk != 0);
+  kbc_collide_m<R, FM, true, S>(f, m[0], R(1) + m[0], m[1], m[2], m[3], beta_c, dux, duy, duz, lbgk != 0);
   store_node<S, R>(pc, fout_c, __ldg(ex_node + k), f);
 }
 
@@ -507,7 +507,7 @@ __global__ void k_moments(PatchDev p, const S* __restrict__ fin, void* rho_o, vo
     vals[1] = ux + R(0.5) * dux;
     vals[2] = uy + R(0.5) * duy;
     vals[3] = uz + R(0.5) * duz;
-    if (gamma_o) vals[4] = kbc_collide<R, 0>(f, beta, R(0), R(0), R(0), lbgk != 0);
+    if (gamma_o) vals[4] = kbc_collide<R, 0, S>(f, beta, R(0), R(0), R(0), lbgk != 0);
   }
   if (dtype == 1) {
     if (rho_o) stv<double>(rho_o, d, vals[0]);
@@ -558,7 +558,7 @@ __global__ void __launch_bounds__(128) k_gamma_blocks(PatchDev p, const S* __res
       R f[27];
       if (t == T_BULK) pull_bulk<S, R>(p, fin, x, y, z, f);
       else pull_generic<S, R>(p, fin, x, y, z, f, status);
-      const R gamma = kbc_collide<R, 0>(f, beta, R(0), R(0), R(0), lbgk != 0);
+      const R gamma = kbc_collide<R, 0, S>(f, beta, R(0), R(0), R(0), lbgk != 0);
       dev = (float)fabs((double)gamma - 2.0);
     }
   }

@@ -417,7 +417,7 @@ __global__ void __launch_bounds__(BX + 32, MINB) k_sc_tma(const __grid_constant_
     }
     __syncwarp();
     if (lane == 0) mbar_arrive(&empty[s]);  // this warp is done with stage s
-    if (x < p.dim[0] && !fixed) kbc_collide<R, FM>(f, E.beta, E.du[0], E.du[1], E.du[2], b.lbgk != 0);
+    if (x < p.dim[0] && !fixed) kbc_collide<R, FM, S>(f, E.beta, E.du[0], E.du[1], E.du[2], b.lbgk != 0);
     // this warp's output segment in stage o: wait until the stores that last
     // used it have read it, fill it, store it
     const int o = k % C::DO;
@@ -626,8 +626,9 @@ __global__ void __launch_bounds__(NP * 64, MINB) k_sc_tma2(const __grid_constant
     {
       F2 rho_t, rho, ux, uy, uz;
       macro_v<F2>(f, rho_t, rho, ux, uy, uz);
-      kbc_collide_v<F2, FM>(f, rho_t, rho, ux, uy, uz, F2(E.beta), F2(E.du[0]), F2(E.du[1]), F2(E.du[2]),
-                            E.du[0] != 0.0f, E.du[1] != 0.0f, E.du[2] != 0.0f, b.lbgk != 0);
+      kbc_collide_v<F2, FM, false, (sizeof(S) > 2)>(f, rho_t, rho, ux, uy, uz, F2(E.beta), F2(E.du[0]),
+                                                    F2(E.du[1]), F2(E.du[2]), E.du[0] != 0.0f, E.du[1] != 0.0f,
+                                                    E.du[2] != 0.0f, b.lbgk != 0);
     }
     if ((fl & 1) && lo_edge) {
       // fixed inlet node: keeps its populations
@@ -673,7 +674,7 @@ __global__ void __launch_bounds__(128) k_sc_tiles(PatchDev p, const S* __restric
   R f[27];
   if (ty == T_BULK) pull_bulk<S, R>(p, fin, x, y, z, f);
   else pull_generic<S, R, true>(p, fin, x, y, z, f, status);
-  kbc_collide<R, FM>(f, beta, dux, duy, duz, lbgk != 0);
+  kbc_collide<R, FM, S>(f, beta, dux, duy, duz, lbgk != 0);
   unroll<27>([&](auto I) {
     constexpr int i = decltype(I)::value;
     Stor<S>::st(fout + (long long)i * p.plane + own, f[i]);
@@ -693,7 +694,7 @@ __global__ void __launch_bounds__(128) k_sc_nodes(PatchDev p, const S* __restric
   const int z = (int)(own / ((long long)p.nxp * p.dim[1]));
   R f[27];
   pull_generic<S, R, true>(p, fin, x, y, z, f, status);
-  kbc_collide<R, FM>(f, beta, dux, duy, duz, lbgk != 0);
+  kbc_collide<R, FM, S>(f, beta, dux, duy, duz, lbgk != 0);
   unroll<27>([&](auto I) {
     constexpr int i = decltype(I)::value;
     Stor<S>::st(fout + (long long)i * p.plane + own, f[i]);
