@@ -23,32 +23,123 @@ struct ThState {
   R T_d;    // T - T0
 };
 
+// Column sums along z of a population set (index c_x + 1, c_y + 1):
+// z0 = sum, z1 = sum of c_z, z2 = sum of c_z^2.  The moments of a set are sums
+// of these 27 values, which they share: 66 additions for the density, momentum
+// and second moments of f, and 49 for the energy and flux of g, against 129 and
+// 77 population by population.
 template <typename R>
-__device__ __forceinline__ void thermal_state(const R (&f)[27], const R (&g)[27], ThState<R>& s) {
-  macro(f, s.rho_t, s.rho, s.ux, s.uy, s.uz);
-  R e[3] = {0, 0, 0};
-  unroll<27>([&](auto I) {
-    constexpr int i = decltype(I)::value;
-    e[CZ(i) + 1] += g[i];
-  });
-  s.e_t = (e[0] + e[2]) + e[1];
-  // T = (2E - u^2)/3 with 2E = (1 + e_t)/rho  =>  T - 1/3 = ((e_t - rho_t)/rho - u^2)/3
+struct ZSums {
+  R z0[3][3], z1[3][3], z2[3][3];
+  template <typename Get>
+  __device__ __forceinline__ explicit ZSums(Get&& get) {
+    unroll<9>([&](auto J) {
+      constexpr int j = decltype(J)::value, a = j % 3, b = j / 3;
+      const R lo = get(std::integral_constant<int, j>{}), mid = get(std::integral_constant<int, j + 9>{}),
+              hi = get(std::integral_constant<int, j + 18>{});
+      z2[a][b] = lo + hi;
+      z1[a][b] = hi - lo;
+      z0[a][b] = z2[a][b] + mid;
+    });
+  }
+  // sum and first moments
+  __device__ __forceinline__ void low(R& m, R (&j)[3]) const {
+    const R x0 = (z0[0][0] + z0[0][2]) + z0[0][1], x2 = (z0[2][0] + z0[2][2]) + z0[2][1];
+    const R x1 = (z0[1][0] + z0[1][2]) + z0[1][1];
+    m = (x0 + x2) + x1;
+    j[0] = x2 - x0;
+    j[1] = ((z0[0][2] + z0[2][2]) + z0[1][2]) - ((z0[0][0] + z0[2][0]) + z0[1][0]);
+    j[2] = (((z1[0][0] + z1[0][2]) + z1[0][1]) + ((z1[2][0] + z1[2][2]) + z1[2][1])) +
+           ((z1[1][0] + z1[1][2]) + z1[1][1]);
+  }
+  // second moments xx, yy, zz, xy, xz, yz
+  __device__ __forceinline__ void second(R (&P)[6]) const {
+    P[0] = ((z0[0][0] + z0[0][2]) + z0[0][1]) + ((z0[2][0] + z0[2][2]) + z0[2][1]);
+    P[1] = ((z0[0][2] + z0[2][2]) + z0[1][2]) + ((z0[0][0] + z0[2][0]) + z0[1][0]);
+    P[2] = (((z2[0][0] + z2[0][2]) + z2[0][1]) + ((z2[2][0] + z2[2][2]) + z2[2][1])) +
+           ((z2[1][0] + z2[1][2]) + z2[1][1]);
+    P[3] = (z0[0][0] + z0[2][2]) - (z0[2][0] + z0[0][2]);
+    P[4] = ((z1[2][0] + z1[2][2]) + z1[2][1]) - ((z1[0][0] + z1[0][2]) + z1[0][1]);
+    P[5] = ((z1[0][2] + z1[2][2]) + z1[1][2]) - ((z1[0][0] + z1[2][0]) + z1[1][0]);
+  }
+};
+
+// (rho, u) from the moments of f, 2 rho E from the sum of g:
+// T = (2E - u^2)/3 with 2E = (1 + e_t)/rho  =>  T - 1/3 = ((e_t - rho_t)/rho - u^2)/3
+template <typename R>
+__device__ __forceinline__ void thermal_state(R rho_t, const R (&j)[3], R e_t, ThState<R>& s) {
+  s.rho_t = rho_t;
+  s.rho = R(1) + rho_t;
+  const R ir = rcp_fast(s.rho);
+  s.ux = j[0] * ir;
+  s.uy = j[1] * ir;
+  s.uz = j[2] * ir;
+  s.e_t = e_t;
   const R u2 = s.ux * s.ux + s.uy * s.uy + s.uz * s.uz;
-  s.T_d = (fdiv(s.e_t - s.rho_t, s.rho) - u2) * R(1.0 / 3.0);
+  s.T_d = ((e_t - rho_t) * ir - u2) * R(1.0 / 3.0);
 }
 
-// g^eq - W_i c_i^2 for (rho, u, 2 rho E); see the header comment.
 template <typename R>
-__device__ __forceinline__ void geq_dev(R rho_t, R rho, R ux, R uy, R uz, R e_t, R (&ge)[27]) {
+__device__ __forceinline__ void thermal_state(const R (&f)[27], const R (&g)[27], ThState<R>& s) {
+  R rho_t, j[3], e_t, q[3];
+  ZSums<R>([&](auto I) { return f[decltype(I)::value]; }).low(rho_t, j);
+  ZSums<R>([&](auto I) { return g[decltype(I)::value]; }).low(e_t, q);
+  thermal_state(rho_t, j, e_t, s);
+}
+
+// c_i . v without the zero components (a product with a zero constant is not
+// folded away)
+template <int i, typename R>
+__device__ __forceinline__ R cdot(R x, R y, R z) {
+  R r = 0;
+  bool first = true;
+  auto add = [&](int c, R v) {
+    if (c == 0) return;
+    r = first ? (c > 0 ? v : -v) : (c > 0 ? r + v : r - v);
+    first = false;
+  };
+  add(CX(i), x);
+  add(CY(i), y);
+  add(CZ(i), z);
+  return r;
+}
+
+// Grad-form equilibrium g^eq - W_i c_i^2 for (rho, u, 2 rho E) (see the header
+// comment of thermal.cu), with an extra first moment:
+//   W_i (e~ + rho~ (c_i^2 - 1) + c_i . (a1 u + V) + a2 ((c_i . u)^2 - u^2/3)),
+// given to put(I, value) population by population.  The terms even in c_i are
+// the same for i and its opposite and the odd ones change sign, so a pair takes
+// them once: about 6 operations a population against 14.
+template <typename R, typename Put>
+__device__ __forceinline__ void geq_terms(R rho_t, R rho, R ux, R uy, R uz, R e_t, R Vx, R Vy, R Vz, Put&& put) {
   const R E2 = R(1) + e_t;
   const R u2 = ux * ux + uy * uy + uz * uz;
   const R a1 = R(3) * (E2 + R(2.0 / 3.0) * rho);
   const R a2 = R(4.5) * (E2 + R(4.0 / 3.0) * rho);
-  unroll<27>([&](auto I) {
-    constexpr int i = decltype(I)::value;
-    const R cu = R(CX(i)) * ux + R(CY(i)) * uy + R(CZ(i)) * uz;
-    ge[i] = R(WI(i)) * (e_t + rho_t * R(C2<i>() - 1) + a1 * cu + a2 * (cu * cu - u2 * R(1.0 / 3.0)));
+  const R Yx = a1 * ux + Vx, Yy = a1 * uy + Vy, Yz = a1 * uz + Vz;
+  const R e0 = e_t - a2 * u2 * R(1.0 / 3.0);
+  // even part by c_i^2 (which is also the weight class)
+  R ev[4], av[4];
+  constexpr double WK[4] = {8.0 / 27.0, 2.0 / 27.0, 1.0 / 54.0, 1.0 / 216.0};
+#pragma unroll
+  for (int k = 0; k < 4; ++k) {
+    ev[k] = R(WK[k]) * (e0 + rho_t * R(k - 1));
+    av[k] = R(WK[k]) * a2;
+  }
+  put(std::integral_constant<int, 13>{}, ev[0]);
+  unroll<13>([&](auto J) {
+    constexpr int i = 26 - decltype(J)::value, k = C2<i>();  // the pair (i, 26 - i)
+    const R cu = cdot<i>(ux, uy, uz);
+    const R even = ev[k] + av[k] * cu * cu;
+    const R odd = R(WK[k]) * cdot<i>(Yx, Yy, Yz);
+    put(std::integral_constant<int, i>{}, even + odd);
+    put(std::integral_constant<int, 26 - i>{}, even - odd);
   });
+}
+
+template <typename R>
+__device__ __forceinline__ void geq_dev(R rho_t, R rho, R ux, R uy, R uz, R e_t, R (&ge)[27]) {
+  geq_terms<R>(rho_t, rho, ux, uy, uz, e_t, R(0), R(0), R(0), [&](auto I, R v) { ge[decltype(I)::value] = v; });
 }
 
 // Non-equilibrium pressure tensor P1 = sum c c (f - f^eq) from f and its equilibrium.
@@ -70,12 +161,12 @@ __device__ __forceinline__ void p1_tensor(const R (&f)[27], const R (&fe)[27], R
 // W_i c_i . V / T0 for a vector V
 template <int i, typename R>
 __device__ __forceinline__ R wcv3(R vx, R vy, R vz) {
-  return R(3.0 * WI(i)) * (R(CX(i)) * vx + R(CY(i)) * vy + R(CZ(i)) * vz);
+  return R(3.0 * WI(i)) * cdot<i>(vx, vy, vz);
 }
 
 // One thermal collision of deviation populations: f in place, g read through
 // gget(I) (the pre-collision g_i, any number of times) and written through
-// gput(I, g'_i) once per population after every read; returns gamma.
+// gput(I, g'_i) once per population after its last read; returns gamma.
 // Pr <= 1: f* = f^eq and g* carries q - 2 u.(P - P^eq) (Table I); Pr > 1:
 // f* - f^eq is the Grad term W_i (P - P^eq)_ab (c_ia c_ib - T0 d_ab)/(2 T0^2)
 // and g* carries q^eq + 2 u.(P - P^eq), with the closed-form P^eq.  The g
@@ -83,39 +174,17 @@ __device__ __forceinline__ R wcv3(R vx, R vy, R vz) {
 template <typename R, typename GGet, typename GPut>
 __device__ __forceinline__ R thermal_collide_acc(R (&f)[27], GGet&& gget, GPut&& gput, R beta, R beta1, R glam,
                                                  R tref_d, bool lbgk, bool pr_gt1) {
+  // moments of the pre-collision state: q = sum c g, P - P^eq = P~ + T0 d - rho T0 d - rho u u
   ThState<R> s;
-  macro(f, s.rho_t, s.rho, s.ux, s.uy, s.uz);
+  R P[6], q[3];
   {
-    R e[3] = {0, 0, 0};
-    unroll<27>([&](auto I) {
-      constexpr int i = decltype(I)::value;
-      e[CZ(i) + 1] += gget(I);
-    });
-    s.e_t = (e[0] + e[2]) + e[1];
-    // T = (2E - u^2)/3 with 2E = (1 + e_t)/rho  =>  T - 1/3 = ((e_t - rho_t)/rho - u^2)/3
-    const R u2 = s.ux * s.ux + s.uy * s.uy + s.uz * s.uz;
-    s.T_d = (fdiv(s.e_t - s.rho_t, s.rho) - u2) * R(1.0 / 3.0);
+    R rho_t, j[3], e_t;
+    const ZSums<R> zf([&](auto I) { return f[decltype(I)::value]; });
+    zf.low(rho_t, j);
+    zf.second(P);
+    ZSums<R>(gget).low(e_t, q);
+    thermal_state(rho_t, j, e_t, s);
   }
-  // pre-collision moments: P - P^eq = P~ + T0 d - rho T0 d - rho u u, q = sum c g
-  R P[6] = {0, 0, 0, 0, 0, 0}, q[3] = {0, 0, 0};
-  unroll<27>([&](auto I) {
-    constexpr int i = decltype(I)::value;
-    if constexpr (CX(i) != 0) P[0] += f[i];
-    if constexpr (CY(i) != 0) P[1] += f[i];
-    if constexpr (CZ(i) != 0) P[2] += f[i];
-    if constexpr (CX(i) * CY(i) != 0) P[3] += R(CX(i) * CY(i)) * f[i];
-    if constexpr (CX(i) * CZ(i) != 0) P[4] += R(CX(i) * CZ(i)) * f[i];
-    if constexpr (CY(i) * CZ(i) != 0) P[5] += R(CY(i) * CZ(i)) * f[i];
-  });
-  unroll<27>([&](auto I) {
-    constexpr int i = decltype(I)::value;
-    if constexpr (CX(i) != 0 || CY(i) != 0 || CZ(i) != 0) {
-      const R gi = gget(I);
-      if constexpr (CX(i) != 0) q[0] += R(CX(i)) * gi;
-      if constexpr (CY(i) != 0) q[1] += R(CY(i)) * gi;
-      if constexpr (CZ(i) != 0) q[2] += R(CZ(i)) * gi;
-    }
-  });
   const R u[3] = {s.ux, s.uy, s.uz};
   const R rt3 = s.rho_t * R(1.0 / 3.0);
   const R Pd[3][3] = {{P[0] - rt3 - s.rho * u[0] * u[0], P[3] - s.rho * u[0] * u[1], P[4] - s.rho * u[0] * u[2]},
@@ -128,19 +197,13 @@ __device__ __forceinline__ R thermal_collide_acc(R (&f)[27], GGet&& gget, GPut&&
     const R Pu2 = R(2) * (Pd[a][0] * u[0] + Pd[a][1] * u[1] + Pd[a][2] * u[2]);
     X[a] = pr_gt1 ? Pu2 : q[a] - qc * u[a] - Pu2;
   }
-  // g^eq - W_i c_i^2 for (rho, u, 2 rho E) (geq_dev), population by population
+  // g' = g + 2 beta (g^eq + (1 - beta1/beta)(g* - g^eq) - g), the quasi-equilibrium
+  // as an extra first moment of the Grad form
   {
-    const R E2 = R(1) + s.e_t;
-    const R u2 = s.ux * s.ux + s.uy * s.uy + s.uz * s.uz;
-    const R a1 = R(3) * (E2 + R(2.0 / 3.0) * s.rho);
-    const R a2 = R(4.5) * (E2 + R(4.0 / 3.0) * s.rho);
-    const R b2 = R(2) * beta, b12 = R(2) * (beta - beta1);
-    unroll<27>([&](auto I) {
-      constexpr int i = decltype(I)::value;
-      const R cu = R(CX(i)) * s.ux + R(CY(i)) * s.uy + R(CZ(i)) * s.uz;
-      const R ge = R(WI(i)) * (s.e_t + s.rho_t * R(C2<i>() - 1) + a1 * cu + a2 * (cu * cu - u2 * R(1.0 / 3.0)));
+    const R b2 = R(2) * beta, r3 = R(3) * fdiv(beta - beta1, beta);
+    geq_terms<R>(s.rho_t, s.rho, s.ux, s.uy, s.uz, s.e_t, r3 * X[0], r3 * X[1], r3 * X[2], [&](auto I, R ge) {
       const R gi = gget(I);
-      gput(I, gi + b2 * (ge - gi) + b12 * wcv3<i>(X[0], X[1], X[2]));
+      gput(I, gi + b2 * (ge - gi));
     });
   }
   const R duz = glam * (s.T_d - tref_d);
@@ -148,18 +211,22 @@ __device__ __forceinline__ R thermal_collide_acc(R (&f)[27], GGet&& gget, GPut&&
   const R gamma = kbc_collide_m<R, 4>(f, s.rho_t, s.rho, s.ux, s.uy, s.uz, beta, R(0), R(0), duz, lbgk);
   if (pr_gt1) {
     // 2 (beta - beta1)(f* - f^eq) at T0 = 1/3: 9 (beta - beta1) W_i Pd_ab (c_ia c_ib - d_ab / 3)
+    // even in c_i: once per pair of opposite directions
     const R k9 = R(9) * (beta - beta1);
     const R tr3 = (Pd[0][0] + Pd[1][1] + Pd[2][2]) * R(1.0 / 3.0);
-    unroll<27>([&](auto I) {
-      constexpr int i = decltype(I)::value;
+    const R xy = R(2) * Pd[0][1], xz = R(2) * Pd[0][2], yz = R(2) * Pd[1][2];
+    unroll<14>([&](auto J) {
+      constexpr int i = 26 - decltype(J)::value;
       R v = -tr3;
       if constexpr (CX(i) != 0) v += Pd[0][0];
       if constexpr (CY(i) != 0) v += Pd[1][1];
       if constexpr (CZ(i) != 0) v += Pd[2][2];
-      if constexpr (CX(i) * CY(i) != 0) v += R(2 * CX(i) * CY(i)) * Pd[0][1];
-      if constexpr (CX(i) * CZ(i) != 0) v += R(2 * CX(i) * CZ(i)) * Pd[0][2];
-      if constexpr (CY(i) * CZ(i) != 0) v += R(2 * CY(i) * CZ(i)) * Pd[1][2];
-      f[i] += k9 * R(WI(i)) * v;
+      if constexpr (CX(i) * CY(i) != 0) v += R(CX(i) * CY(i)) * xy;
+      if constexpr (CX(i) * CZ(i) != 0) v += R(CX(i) * CZ(i)) * xz;
+      if constexpr (CY(i) * CZ(i) != 0) v += R(CY(i) * CZ(i)) * yz;
+      const R w = k9 * R(WI(i));
+      f[i] += w * v;
+      if constexpr (i != 13) f[26 - i] += w * v;
     });
   }
   return gamma;
