@@ -482,44 +482,41 @@ cudaError_t launch_transfer(int storage, const PatchDev& p, void* f0, void* f1, 
   });
 }
 
-template <typename V>
-__device__ __forceinline__ void stv(void* p, long long i, double v) {
-  ((V*)p)[i] = (V)v;
-}
-
-template <typename S, typename R>
-__global__ void k_moments(PatchDev p, const S* __restrict__ fin, void* rho_o, void* u_o, void* gamma_o, int dtype,
-                          R beta, R dux, R duy, R duz, int lbgk) {
-  const int x = blockIdx.x * blockDim.x + threadIdx.x;
-  const int y = blockIdx.y, z = blockIdx.z;
+// One thread per stored node, rows packed end to end (x fastest, padding
+// included), so that short rows do not leave most of a block idle.  O is the
+// type of the outputs: in FP32 no operation is FP64.  The pass reads its
+// populations once and should run at the copy bandwidth; FP64 sums and
+// conversions of the four outputs had bound it instead (five patches of the
+// 256 x 64 x 128 channel, FP32: 468 us against 552, 440 at the copy rate).
+template <typename S, typename R, typename O>
+__global__ void __launch_bounds__(128) k_moments(PatchDev p, const S* __restrict__ fin, O* __restrict__ rho_o,
+                                                 O* __restrict__ u_o, O* __restrict__ gamma_o, R beta, R dux, R duy,
+                                                 R duz, int lbgk) {
+  const long long own = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+  if (own >= p.plane) return;
+  const unsigned row = (unsigned)own / (unsigned)p.nxp;  // node indices fit 32 bits
+  const int x = (int)((unsigned)own - row * (unsigned)p.nxp);
   if (x >= p.dim[0]) return;
-  const long long own = node_index(p, x, y, z);
-  const long long d = ((long long)z * p.dim[1] + y) * p.dim[0] + x;
+  const long long d = (long long)row * p.dim[0] + x;
   const long long nd = (long long)p.dim[0] * p.dim[1] * p.dim[2];
   const uint8_t t = p.type[own];
-  double vals[5] = {0, 0, 0, 0, 0};
+  O vals[5] = {0, 0, 0, 0, 0};
   if (t != T_SKIP && t != T_SOLID) {
     R f[27];
     load_node<S, R>(p, fin, own, f);
     R rho_t, rho, ux, uy, uz;
     macro(f, rho_t, rho, ux, uy, uz);
-    vals[0] = (double)rho_t + 1.0;
-    vals[1] = ux + R(0.5) * dux;
-    vals[2] = uy + R(0.5) * duy;
-    vals[3] = uz + R(0.5) * duz;
-    if (gamma_o) vals[4] = kbc_collide<R, 0, S>(f, beta, R(0), R(0), R(0), lbgk != 0);
+    using W = decltype(R() + O());  // the wider of the two
+    vals[0] = (O)((W)rho_t + W(1));
+    vals[1] = (O)(ux + R(0.5) * dux);
+    vals[2] = (O)(uy + R(0.5) * duy);
+    vals[3] = (O)(uz + R(0.5) * duz);
+    if (gamma_o) vals[4] = (O)kbc_collide<R, 0, S>(f, beta, R(0), R(0), R(0), lbgk != 0);
   }
-  if (dtype == 1) {
-    if (rho_o) stv<double>(rho_o, d, vals[0]);
-    if (u_o)
-      for (int a = 0; a < 3; ++a) stv<double>(u_o, a * nd + d, vals[1 + a]);
-    if (gamma_o) stv<double>(gamma_o, d, vals[4]);
-  } else {
-    if (rho_o) stv<float>(rho_o, d, vals[0]);
-    if (u_o)
-      for (int a = 0; a < 3; ++a) stv<float>(u_o, a * nd + d, vals[1 + a]);
-    if (gamma_o) stv<float>(gamma_o, d, vals[4]);
-  }
+  if (rho_o) rho_o[d] = vals[0];
+  if (u_o)
+    for (int a = 0; a < 3; ++a) u_o[a * nd + d] = vals[1 + a];
+  if (gamma_o) gamma_o[d] = vals[4];
 }
 
 cudaError_t launch_moments(int storage, const PatchDev& p, const void* fin, void* rho, void* u, void* gamma,
@@ -527,9 +524,14 @@ cudaError_t launch_moments(int storage, const PatchDev& p, const void* fin, void
   return dispatch(storage, [&](auto ts, auto tr) {
     using S = typename decltype(ts)::type;
     using R = typename decltype(tr)::type;
-    dim3 block(128), grid((p.dim[0] + 127) / 128, p.dim[1], p.dim[2]);
-    k_moments<S, R><<<grid, block, 0, st>>>(p, (const S*)fin, rho, u, gamma, dtype, (R)beta, (R)F.du[0],
-                                            (R)F.du[1], (R)F.du[2], lbgk);
+    const unsigned grid = (unsigned)((p.plane + 127) / 128);
+    auto go = [&](auto o) {
+      using O = decltype(o);
+      k_moments<S, R, O><<<grid, 128, 0, st>>>(
+          p, (const S*)fin, (O*)rho, (O*)u, (O*)gamma, (R)beta, (R)F.du[0], (R)F.du[1], (R)F.du[2], lbgk);
+    };
+    if (dtype == 1) go(double(0));
+    else go(float(0));
     return cudaGetLastError();
   });
 }
