@@ -157,20 +157,26 @@ struct AxisV {
   V s, B;
 };
 
+// axis_eq_den: the two denominators of an axis, den[0] = (1 - u)(2u + s) and
+// den[1] = (s + 1) A; axis_eq_r: its factors from their reciprocals.
 template <typename V>
-__device__ __forceinline__ void axis_eq_v(V u, AxisV<V>& a, bool want_inverse) {
+__device__ __forceinline__ void axis_eq_den(V u, AxisV<V>& a, V (&den)[2]) {
+  const V one = K<V>(1.0), two = K<V>(2.0);
+  a.s = vsqrt1(vfma(K<V>(3.0), u * u, one));
+  den[0] = (one - u) * vfma(two, u, a.s);
+  den[1] = (a.s + one) * (two - a.s);
+}
+
+template <typename V>
+__device__ __forceinline__ void axis_eq_r(V u, V r1, V r2, AxisV<V>& a, bool want_inverse) {
   const V one = K<V>(1.0), two = K<V>(2.0), three = K<V>(3.0);
   const V u2 = u * u;
-  const V s = vsqrt1(vfma(three, u2, one));
   const V om = one - u;
-  const V tus = vfma(two, u, s);
-  const V r1 = vrcp(om * tus);
+  const V tus = vfma(two, u, a.s);
   const V i1mu = tus * r1, i2us = om * r1;
-  const V sp1 = s + one, A = two - s;
-  const V r2 = vrcp(sp1 * A);
+  const V sp1 = a.s + one, A = two - a.s;
   const V e = (three * u2) * (A * r2);
   const V e2 = e + e;
-  a.s = s;
   a.B = tus * i1mu;
   a.d[1] = -e;
   a.d[2] = vfma(u, vfma(-three, u, three - e2), e2) * i1mu;
@@ -181,6 +187,39 @@ __device__ __forceinline__ void axis_eq_v(V u, AxisV<V>& a, bool want_inverse) {
     a.ig[1] = K<V>(1.5) * iA;
     a.ig[2] = iA6 * (om * i2us);
     a.ig[0] = iA6 * a.B;
+  }
+}
+
+template <typename V>
+__device__ __forceinline__ void axis_eq_v(V u, AxisV<V>& a, bool want_inverse) {
+  V den[2];
+  axis_eq_den(u, a, den);
+  axis_eq_r(u, vrcp(den[0]), vrcp(den[1]), a, want_inverse);
+}
+
+// The three axes of a node.  FP64 takes the six reciprocals from that of the
+// product of the denominators (each near 1 or 2): a division there costs about
+// as many operations of the slow FP64 pipe as the fifteen products that
+// replace five of them do not; the FP32 reciprocal is one instruction of
+// another pipe.
+template <typename V>
+__device__ __forceinline__ void axes_eq_v(V ux, V uy, V uz, AxisV<V>& ex, AxisV<V>& ey, AxisV<V>& ez,
+                                          bool want_inverse) {
+  if constexpr (std::is_same<V, double>::value) {
+    double x[2], y[2], z[2];
+    axis_eq_den(ux, ex, x);
+    axis_eq_den(uy, ey, y);
+    axis_eq_den(uz, ez, z);
+    const double px = x[0] * x[1], py = y[0] * y[1], pz = z[0] * z[1], pxy = px * py;
+    const double r = vrcp(pxy * pz);
+    const double rz = r * pxy, rxy = r * pz, rx = rxy * py, ry = rxy * px;
+    axis_eq_r(ux, rx * x[1], rx * x[0], ex, want_inverse);
+    axis_eq_r(uy, ry * y[1], ry * y[0], ey, want_inverse);
+    axis_eq_r(uz, rz * z[1], rz * z[0], ez, want_inverse);
+  } else {
+    axis_eq_v(ux, ex, want_inverse);
+    axis_eq_v(uy, ey, want_inverse);
+    axis_eq_v(uz, ez, want_inverse);
   }
 }
 
@@ -320,9 +359,7 @@ template <typename V, int FM, bool DF = false, bool TAB = true>
 __device__ __forceinline__ V kbc_collide_v(V (&f)[27], V rho_t, V rho, V ux, V uy, V uz, V beta, V dux, V duy,
                                            V duz, bool du_x, bool du_y, bool du_z, bool lbgk) {
   AxisV<V> ex, ey, ez;
-  axis_eq_v<V>(ux, ex, !lbgk);
-  axis_eq_v<V>(uy, ey, !lbgk);
-  axis_eq_v<V>(uz, ez, !lbgk);
+  axes_eq_v<V>(ux, uy, uz, ex, ey, ez, !lbgk);
   // f becomes df = f - f^eq
   if constexpr (!DF && !TAB) {
     const EqClasses<V> T(rho_t, rho, ex.d, ey.d);
@@ -409,8 +446,14 @@ __device__ __forceinline__ V kbc_collide_v(V (&f)[27], V rho_t, V rho, V ux, V u
     const V w0 = irho * ez.ig[0], w1 = irho * ez.ig[1], w2 = irho * ez.ig[2];
     const V sh = vfma(w1, shl[1], vfma(w0, shl[0], w2 * shl[2]));
     const V hh = vfma(w1, hhl[1], vfma(w0, hhl[0], w2 * hhl[2]));
-    const V ib = vrcp(beta);
-    const V g = ib - (K<V>(2.0) - ib) * (sh * vrcp(hh));
+    V ib, ihh;
+    if constexpr (std::is_same<V, double>::value) {
+      const V r = vrcp(beta * hh);  // hh = 0: not used below
+      ib = hh * r, ihh = beta * r;
+    } else {
+      ib = vrcp(beta), ihh = vrcp(hh);
+    }
+    const V g = ib - (K<V>(2.0) - ib) * (sh * ihh);
     gamma = vsel_gt(hh, K<V>(1e-30) * rho * rho, g, gamma);
   }
   // f' = f^eq(rho, u + du) + (1 - beta gamma) df + beta (gamma - 2) ds: the
