@@ -412,6 +412,11 @@ lbm_status run_instant(lbm_grid* g, int k) {
                                                             (int64_t)p.fix_nodes[odd].size(), TL, status_ptr(g),
                                                             g->stream);
                                 if (!e)
+                                  e = lbmk::launch_th_nodes(storage, pv, fin, gin, fout, gout,
+                                                            at<uint32_t>(g, p.off_dense_nodes[odd]),
+                                                            (int64_t)p.dense_nodes[odd].size(), TL, status_ptr(g),
+                                                            g->stream);
+                                if (!e)
                                   e = lbmk::launch_th_tiles(storage, pv, fin, gin, fout, gout,
                                                             at<uint32_t>(g, p.off_tiles_mixed[odd]),
                                                             (int64_t)p.tiles_mixed[odd].size(), (int)p.ntx, TL, odd,
@@ -426,8 +431,12 @@ lbm_status run_instant(lbm_grid* g, int k) {
             timed(g, 0, lev, g->timing ? count_types(p, odd) - p.n_tma[odd] : 0.0,
                   [&] {
                     cudaError_t e = lbmk::launch_sc_nodes(storage, pv, fin, fout, at<uint32_t>(g, p.off_fix_nodes[odd]),
-                                              (int64_t)p.fix_nodes[odd].size(), p.beta, F, lbgk, status_ptr(g),
-                                              rest);
+                                              (int64_t)p.fix_nodes[odd].size(), p.beta, F, lbgk, false,
+                                              status_ptr(g), rest);
+                    if (!e)
+                      e = lbmk::launch_sc_nodes(storage, pv, fin, fout, at<uint32_t>(g, p.off_dense_nodes[odd]),
+                                                (int64_t)p.dense_nodes[odd].size(), p.beta, F, lbgk, true,
+                                                status_ptr(g), rest);
                     if (e) return e;
                     return lbmk::launch_sc_tiles(storage, pv, fin, fout, at<uint32_t>(g, p.off_tiles_mixed[odd]),
                                                  (int64_t)p.tiles_mixed[odd].size(), (int)p.ntx, p.beta, F, odd,
@@ -686,6 +695,7 @@ lbm_status lbm_grid_bind(lbm_grid_t g, void* dev_ptr, size_t bytes, void* cuda_s
       if (!e) e = up(p.off_tiles_half[k], p.tiles_half[k].data(), 8 * p.tiles_half[k].size());
     for (int k = 0; k < 2; ++k) {
       if (!e) e = up(p.off_tiles_mixed[k], p.tiles_mixed[k].data(), 4 * p.tiles_mixed[k].size());
+      if (!e) e = up(p.off_dense_nodes[k], p.dense_nodes[k].data(), 4 * p.dense_nodes[k].size());
       if (!e) e = up(p.off_fix_nodes[k], p.fix_nodes[k].data(), 4 * p.fix_nodes[k].size());
       if (!e) e = up(p.off_tiles_all[k], p.tiles_all[k].data(), 4 * p.tiles_all[k].size());
     }

@@ -56,6 +56,9 @@ struct HostPatch {
   std::vector<uint32_t> tiles_mixed[2];  // other tiles with nodes to update: [0] even, [1] odd steps
   std::vector<uint32_t> tiles_all[2];    // every tile with nodes to update (thermal model, node by node)
   std::vector<uint32_t> fix_nodes[2];    // nodes of TMA tiles recomputed node by node after the tile pass
+  // every updated node of the patch, for FP64 patches that go node by node (no
+  // tiles then)
+  std::vector<uint32_t> dense_nodes[2];
   double n_tma[2] = {0, 0};              // updated nodes the TMA pass gives (per parity)
   alignas(64) unsigned char tmap[2][128];   // TMA load descriptors of the two population buffers
   alignas(64) unsigned char tmapo[2][128];  // TMA store descriptors
@@ -95,7 +98,7 @@ struct HostPatch {
 
   // device placement (byte offsets into the bound buffer)
   size_t off_f[2]{}, off_g[2]{}, off_type = 0;
-  size_t off_tiles_pure[2]{}, off_tiles_half[2]{}, off_tiles_mixed[2]{}, off_tiles_all[2]{}, off_fix_nodes[2]{};
+  size_t off_tiles_pure[2]{}, off_tiles_half[2]{}, off_tiles_mixed[2]{}, off_tiles_all[2]{}, off_fix_nodes[2]{}, off_dense_nodes[2]{};
   size_t off_ex_node = 0, off_ex_src = 0, off_pt_src = 0, off_use_ptr = 0, off_use_ent = 0;
   size_t off_smp_node = 0, off_smp_kind = 0, off_smp_val = 0, off_cf_parent = 0, off_cf_child = 0;
   size_t off_drag_node = 0, off_drag_mask = 0, off_wq = 0, off_wq_idx = 0;

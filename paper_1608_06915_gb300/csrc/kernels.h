@@ -120,9 +120,11 @@ cudaError_t launch_sc_tma(int storage, const TmaLaunchPatch* ps, int n, int vari
 int sc_tma_variants(int storage);
 // nodes per tile of a variant: 128, or 64 (tmap_in of kind 3, the half-tile list)
 int sc_tma_tile_nodes(int storage, int variant);
-// node-by-node recomputation of listed nodes (after the TMA tile pass)
+// node-by-node stream-collide of listed nodes: fix-up nodes (after the TMA tile
+// pass) or, dense, all updated nodes of a patch without tiles
 cudaError_t launch_sc_nodes(int storage, const PatchDev& p, const void* fin, void* fout, const uint32_t* nodes,
-                            int64_t n, double beta, const Force& F, int lbgk, int* status, cudaStream_t st);
+                            int64_t n, double beta, const Force& F, int lbgk, bool dense, int* status,
+                            cudaStream_t st);
 cudaError_t launch_sc_tiles(int storage, const PatchDev& p, const void* fin, void* fout, const uint32_t* tiles,
                             int64_t ntiles, int ntx, double beta, const Force& F, int odd, int lbgk, int* status,
                             cudaStream_t st);

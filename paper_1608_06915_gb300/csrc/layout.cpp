@@ -475,12 +475,34 @@ std::string build_layout(HostGrid& g) {
       p.tiles_mixed[k].clear();
       p.tiles_all[k].clear();
       p.fix_nodes[k].clear();
+      p.dense_nodes[k].clear();
     }
     struct Rows {
       std::vector<uint64_t> pure[2];
-      std::vector<uint32_t> mixed[2], all[2], fix[2];
+      std::vector<uint32_t> mixed[2], all[2], fix[2], dense[2];
       double ntma[2] = {0, 0};
     };
+    // FP64 is bound by the FP64 pipe, where a warp costs the same whatever its
+    // active lanes, so a patch whose rows leave more than a tenth of the tiles'
+    // lanes idle goes node by node from a packed list (k_sc_nodes): rows of 100
+    // nodes 0.412 ms a step against 0.513, while rows of 128 stay on the tiles.
+    // The thermal model always does, its FP64 tile pass keeps 4 warps per SM:
+    // 40 x 24 x 32 cell 4.67 ms a step against 6.96.
+    bool dense = false;
+    if (g.pop_bytes == 8) {
+      double nodes = 0, lanes = 0;
+      for (int64_t row = 0; row < p.dim[1] * p.dim[2]; ++row)
+        for (int64_t x0 = 0; x0 < p.dim[0]; x0 += 128) {
+          const int64_t n = std::min<int64_t>(128, p.dim[0] - x0);
+          const uint8_t* t = &p.type[row * p.nxp + x0];
+          const auto act = std::count_if(t, t + n, [](uint8_t v) { return v == T_BULK || v == T_BC; });
+          nodes += (double)act;
+          if (act) lanes += (double)((n + 31) / 32 * 32);
+        }
+      // (the tile pass carries an inlet node's populations along)
+      const bool inlet = std::find(p.type.begin(), p.type.end(), (uint8_t)T_INLET) != p.type.end();
+      dense = !inlet && (g.thermal || nodes < 0.9 * lanes);
+    }
     std::vector<Rows> rows(p.dim[2]);
 #pragma omp parallel for schedule(dynamic, 1)
     for (int64_t z = 0; z < p.dim[2]; ++z) {
@@ -506,6 +528,11 @@ std::string build_layout(HostGrid& g) {
             act[0] = t == T_BULK || t == T_BC;
             act[1] = act[0] || t == T_D1;
             if (!act[1]) continue;
+            if (dense) {
+              for (int k = 0; k < 2; ++k)
+                if (act[k]) R.dense[k].push_back((uint32_t)m);
+              continue;
+            }
             for (int k = 0; k < 2; ++k) active[k] += act[k];
             bool regular = true;
             if (t != T_BULK) {
@@ -524,12 +551,8 @@ std::string build_layout(HostGrid& g) {
           const uint32_t id = (uint32_t)((z * p.dim[1] + y) * p.ntx + tx);
           // the TMA path fetches the periodic wrap of x-spanning rows as aligned
           // 16-byte boxes, so rows of any length can take it (a row of one node
-          // would need both wraps at once).  FP64 thermal rows of odd lengths
-          // stay on the node-by-node kernel: that collision is bound by the FP64
-          // pipe, and the tile pass keeps fewer warps on it.
-          const bool edge = tx == 0 || (tx + 1) * 128 >= p.dim[0];
-          const bool wrap_ok = !p.span[0] || !edge || p.dim[0] % 8 == 0 ||
-                               (p.dim[0] >= 2 && !(g.thermal && g.pop_bytes == 8));
+          // would need both wraps at once)
+          const bool wrap_ok = !p.span[0] || p.dim[0] >= 2;
           for (int k = 0; k < 2; ++k) {
             if (active[k] == 0) continue;
             R.all[k].push_back(id);
@@ -562,6 +585,7 @@ std::string build_layout(HostGrid& g) {
         p.tiles_mixed[k].insert(p.tiles_mixed[k].end(), R.mixed[k].begin(), R.mixed[k].end());
         p.tiles_all[k].insert(p.tiles_all[k].end(), R.all[k].begin(), R.all[k].end());
         p.fix_nodes[k].insert(p.fix_nodes[k].end(), R.fix[k].begin(), R.fix[k].end());
+        p.dense_nodes[k].insert(p.dense_nodes[k].end(), R.dense[k].begin(), R.dense[k].end());
       }
   }
   // momentum-exchange links of patches holding solid nodes
@@ -876,6 +900,7 @@ size_t plan_memory(HostGrid& g) {
     p.off_tiles_mixed[1] = take(4 * p.tiles_mixed[1].size());
     p.off_fix_nodes[0] = take(4 * p.fix_nodes[0].size());
     p.off_fix_nodes[1] = take(4 * p.fix_nodes[1].size());
+    for (int k = 0; k < 2; ++k) p.off_dense_nodes[k] = take(4 * p.dense_nodes[k].size());
     p.off_ex_node = take(4 * p.ex_node.size());
     p.off_ex_src = take(4 * p.ex_src.size());
     p.off_pt_src = take(4 * p.pt_src.size());

@@ -45,16 +45,16 @@ cudaError_t launch_sc_tiles(int storage, const PatchDev& p, const void* fin, voi
 }
 
 cudaError_t launch_sc_nodes(int storage, const PatchDev& p, const void* fin, void* fout, const uint32_t* nodes,
-                            int64_t n, double beta, const Force& F, int lbgk, int* status, cudaStream_t st) {
+                            int64_t n, double beta, const Force& F, int lbgk, bool dense, int* status, cudaStream_t st) {
   switch (storage) {
     case LBM_FP64:
-      return sc_nodes_fp64(p, fin, fout, nodes, n, beta, F, lbgk, status, st);
+      return sc_nodes_fp64(p, fin, fout, nodes, n, beta, F, lbgk, dense, status, st);
     case LBM_FP32:
-      return sc_nodes_fp32(p, fin, fout, nodes, n, beta, F, lbgk, status, st);
+      return sc_nodes_fp32(p, fin, fout, nodes, n, beta, F, lbgk, dense, status, st);
     case LBM_FP16_SHIFT:
-      return sc_nodes_fp16(p, fin, fout, nodes, n, beta, F, lbgk, status, st);
+      return sc_nodes_fp16(p, fin, fout, nodes, n, beta, F, lbgk, dense, status, st);
     case LBM_BF16_SHIFT:
-      return sc_nodes_bf16(p, fin, fout, nodes, n, beta, F, lbgk, status, st);
+      return sc_nodes_bf16(p, fin, fout, nodes, n, beta, F, lbgk, dense, status, st);
     default:
       return cudaErrorInvalidValue;
   }

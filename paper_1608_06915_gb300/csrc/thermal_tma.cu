@@ -236,7 +236,9 @@ __global__ void __launch_bounds__(160, ThTmaCfg<R, 1>::MINB) k_th_tma_d(const __
   th_tma_body<R, 1>(m, p, fin, fout, gout, tiles, ntiles, tp, status);
 }
 
-// Nodes of TMA tiles the row rule does not give, recomputed node by node.
+// Listed nodes, a thread each: nodes of TMA tiles the row rule does not give,
+// recomputed after the tile pass, and at FP64 every updated node of a patch
+// (HostPatch::dense_nodes).
 template <typename R>
 __global__ void __launch_bounds__(128) k_th_nodes(PatchDev p, const R* __restrict__ fin, const R* __restrict__ gin,
                                                   R* __restrict__ fout, R* __restrict__ gout,
