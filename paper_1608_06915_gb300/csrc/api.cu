@@ -560,13 +560,13 @@ lbm_status run_instant(lbm_grid* g, int k) {
 // within 1% of the fastest on rows that fill its tiles: 3.23 ms a step against
 // kernel 0's 3.55 on the 256 x 64 x 128 channel, 2.02 against 2.25 on the
 // sphere.  The 64-node tiles take over where they leave a quarter of the lanes
-// fewer idle: 24^3 box 8.2 us against 9.9, 32^3 FP64 two-level box 0.260 ms
-// against 0.275 (kernel 0: 0.444), 27 x 53 x 108 BF16 box 0.067 against 0.079;
-// at equal lanes they lose (20 x 49 x 25 FP64 channel 2.40 against 2.00).  The
-// samples run beside the pass below a million node updates an instant, where
-// the pass leaves the GPU idle (64^3 two-level box, 0.39 M: 0.086 ms against
-// 0.093; reduced curved sphere, 0.5 M: 0.447 against 0.461); the sphere at
-// 4.3 M loses 6% by it.  The thermal model keeps its kernel 0.
+// fewer idle: 24^3 box 8.2 us against 9.9, 27 x 53 x 108 BF16 box 0.067 ms
+// against 0.079; at equal lanes they lose (the channel 3.89 against 3.23, at
+// 101 x 49 x 75 0.921 against 0.914).  The samples run beside the pass below a
+// million node updates an instant, where the pass leaves the GPU idle (64^3
+// two-level box, 0.39 M: 0.086 ms against 0.093; reduced curved sphere, 0.5 M:
+// 0.447 against 0.461); the sphere at 4.3 M loses 6% by it.  The thermal model
+// keeps its kernel 0; FP64 patches without tiles run none of these kernels.
 void default_variant(lbm_grid* g) {
   if (g->hg.thermal) return;
   double l128 = 0, l64 = 0, updates = 0;
