@@ -229,7 +229,10 @@ lbm_status lbm_step(lbm_grid_t g, int64_t n_coarse_steps);
  * Synchronises the bound stream; drops captured step graphs.  Without a call
  * the grid uses the variant a rule on its tiles and size gives (isothermal:
  * kernel 1 or the 64-node tiles, samples beside the pass on small grids;
- * thermal: variant 0).  The paper has no counterpart. */
+ * thermal: variant 0).  A one-level isothermal grid of few tiles (FP32 and
+ * 16-bit storage, no inflow, solids or x walls) runs node by node instead, with
+ * the same results, before and after this call, until lbm_set_variant asks for
+ * a kernel of the tile pass.  The paper has no counterpart. */
 lbm_status lbm_autotune(lbm_grid_t g, int32_t trials, int32_t* chosen, float* ms_per_step, int32_t max_variants,
                         int32_t* n_variants);
 

@@ -59,6 +59,7 @@ struct lbm_grid {
   int wait_sleeps = 1 << 21;  // bound of the TMA passes' stage waits (lbm_wait_limit)
   int device = -1;         // device of the bound buffer
   bool presample = false;  // reconstruction samples beside the TMA pass (lbm_autotune)
+  bool node_pass = false;  // every tile on the node-by-node kernel (small_grid)
   std::vector<Rec> recs;
   std::vector<cudaEvent_t> pool;
   size_t pool_used = 0;
@@ -315,7 +316,7 @@ lbm_status run_instant(lbm_grid* g, int k) {
     }
     if (e) return cuda_check(g, e, "samples");
   }
-  if (!hg.thermal) {
+  if (!hg.thermal && !g->node_pass) {
     // TMA tile pass of every patch stepped at this instant: one persistent
     // launch per 8 patches, whatever their levels and sizes
     // (the 64-node tile variant takes the half-tile lists and their load descriptors)
@@ -424,6 +425,16 @@ lbm_status run_instant(lbm_grid* g, int k) {
                                 return e;
                               }),
                         "thermal stream_collide");
+      } else if (g->node_pass) {
+        st = cuda_check(g,
+                        timed(g, 0, lev, g->timing ? count_types(p, odd) : 0.0,
+                              [&] {
+                                return lbmk::launch_sc_tiles(storage, pv, fin, fout,
+                                                             at<uint32_t>(g, p.off_tiles_all[odd]),
+                                                             (int64_t)p.tiles_all[odd].size(), (int)p.ntx, p.beta, F,
+                                                             odd, lbgk, status_ptr(g), rest);
+                              }),
+                        "stream_collide");
       } else {
         // the nodes the TMA pass does not give: fix-up list, then mixed tiles
         st = cuda_check(
@@ -555,14 +566,39 @@ lbm_status run_instant(lbm_grid* g, int k) {
   return LBM_OK;
 }
 
+// One-level grids of few tiles run node by node (k_sc_tiles over every tile),
+// whichever kernel is chosen for the tile pass, until lbm_set_variant asks for
+// one: at that size a launch is latency, and the tile pass has the longer
+// chain (barriers and descriptors, the stage's loads, the stores of the output
+// stage).  Microseconds per step, node by node against the best tile kernel:
+// FP32 25^3 6.2 / 8.2, 119 x 25 x 24 6.2 / 8.2, 197 x 25 x 25 10.3 / 12.3,
+// 37^3 (1369 tiles) and 181 x 30 x 30 (1800) equal, 43^3 (1849) 11.7 / 11.3,
+// 99 x 60 x 60 (3600) 25.3 / 23.0.  16-bit storage is bound by instruction
+// issue, not by the loads the tiles save, and rows beyond 64 nodes (where the
+// 64-node tiles have no lanes to win) keep the lead longer: FP16 119 x 60 x 60
+// (3600) 20.5 / 22.5, 75^3 (5625) 26.6 / 28.6, 181 x 60 x 60 (7200) 34.0 / 34.9,
+// 197 x 60 x 60 (7200) 38.7 / 36.5; 61^3 (3721, rows of 61) 18.5 / 16.4.
+// Refined grids batch their patches in one tile launch, which is the faster
+// there; at FP64 the packed lists have the short rows.  Grids with fix-up
+// nodes (next to solids, x walls) stay on the tile pass: its fix-up kernel
+// rounds those nodes differently, and all schedules give the same bits.
+bool small_grid(const lbm_grid* g) {
+  const HostGrid& hg = g->hg;
+  if (hg.nlev > 1 || hg.thermal || hg.pop_bytes > 4 || hg.desc.inflow_axis >= 0) return false;
+  const HostPatch& p = hg.P[0];
+  if (!p.fix_nodes[0].empty()) return false;
+  const size_t per_sm = hg.pop_bytes == 2 && p.dim[0] > 64 ? 40 : 12;
+  return p.tiles_all[0].size() <= per_sm * 152;
+}
+
 // The variant a grid runs until lbm_autotune or lbm_set_variant chooses one.
 // Kernel 1 (128-node tiles, two load stages, 4 CTAs per SM) is the faster or
 // within 1% of the fastest on rows that fill its tiles: 3.23 ms a step against
 // kernel 0's 3.55 on the 256 x 64 x 128 channel, 2.02 against 2.25 on the
 // sphere.  The 64-node tiles take over where they leave a quarter of the lanes
-// fewer idle: 24^3 box 8.2 us against 9.9, 27 x 53 x 108 BF16 box 0.067 ms
-// against 0.079; at equal lanes they lose (the channel 3.89 against 3.23, at
-// 101 x 49 x 75 0.921 against 0.914).  The samples run beside the pass below a
+// fewer idle: 27 x 53 x 108 BF16 box 0.067 ms against 0.079; at equal lanes
+// they lose (the channel 3.89 against 3.23, at 101 x 49 x 75 0.921 against
+// 0.914).  The samples run beside the pass below a
 // million node updates an instant, where the pass leaves the GPU idle (64^3
 // two-level box, 0.39 M: 0.086 ms against 0.093; reduced curved sphere, 0.5 M:
 // 0.447 against 0.461); the sphere at 4.3 M loses 6% by it.  The thermal model
@@ -580,6 +616,7 @@ void default_variant(lbm_grid* g) {
   }
   g->variant = l64 <= 0.75 * l128 ? lbmk::sc_tma_variants(g->hg.desc.storage) - 1 : 1;
   g->presample = updates < 1e6 * (double)(1LL << (g->hg.nlev - 1));
+  g->node_pass = small_grid(g);
 }
 
 }  // namespace
@@ -876,6 +913,7 @@ lbm_status lbm_autotune(lbm_grid_t g, int32_t trials, int32_t* chosen, float* ms
   // one untimed step first: the first launches of a kernel pay for loading it
   g->variant = 0;
   g->presample = false;
+  g->node_pass = false;
   lbm_status st = e ? LBM_OK : coarse_step_eager(g);
   g->stepped = true;
   auto trial = [&](int v, int n) {
@@ -911,6 +949,7 @@ lbm_status lbm_autotune(lbm_grid_t g, int32_t trials, int32_t* chosen, float* ms
   if (nv > 1 && ms[second] < ms[best]) best = second;
   g->variant = best % nt;
   g->presample = best >= nt;
+  g->node_pass = small_grid(g);
   g->stepped = true;
   g->drop_graphs();
   if (chosen) *chosen = best;
@@ -927,6 +966,7 @@ lbm_status lbm_set_variant(lbm_grid_t g, int32_t variant) {
   if (variant < 0 || variant >= nv) return fail(g, LBM_ERR_ARG, "variant out of range");
   g->variant = variant % nt;
   g->presample = variant >= nt;
+  g->node_pass = false;
   g->drop_graphs();
   return LBM_OK;
 }

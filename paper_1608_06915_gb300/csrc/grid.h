@@ -54,7 +54,7 @@ struct HostPatch {
   // starts beyond the row is left out), for the 64-node tile variant
   std::vector<uint64_t> tiles_half[2];
   std::vector<uint32_t> tiles_mixed[2];  // other tiles with nodes to update: [0] even, [1] odd steps
-  std::vector<uint32_t> tiles_all[2];    // every tile with nodes to update (thermal model, node by node)
+  std::vector<uint32_t> tiles_all[2];    // every tile with nodes to update (small grids, node by node)
   std::vector<uint32_t> fix_nodes[2];    // nodes of TMA tiles recomputed node by node after the tile pass
   // every updated node of the patch, for FP64 patches that go node by node (no
   // tiles then)

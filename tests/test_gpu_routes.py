@@ -1,0 +1,77 @@
+"""Which kernel a grid's stream-collide runs on, and that each route gives the
+result of the others or of the oracle at the sizes where the rules change
+(GPU).  The route is read from the per-launch timing: "stream_collide_tma" is
+the tile pass, "stream_collide" the node-by-node kernels."""
+import numpy as np
+import pytest
+
+from gpu_util import pop_diff, twin
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _lib():
+    import torch
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_1608_06915_gb300 import build as B
+    B.build()
+
+
+def box(n, walls=(0,) * 6, accel0=(0, 0, 0), boxes=(), solid=None, thermal=None, **more):
+    return dict(name="routes", n=n, periodic=tuple(int(not walls[2 * a]) for a in range(3)), walls=walls,
+                inflow_axis=-1, u_in=(0, 0, 0), boxes=list(boxes), solid=solid, nu0=0.01, accel0=accel0,
+                mirror_lbgk=False, thermal=thermal, **more)
+
+
+def noisy(seed, thermal=False):
+    def fields(x, y, z, p, info):
+        shp = tuple(reversed(info["dim"]))
+        r = np.random.default_rng(seed + p)
+        out = [1.0 + 0.01 * r.uniform(-1, 1, shp), 0.03 * r.uniform(-1, 1, (3,) + shp)]
+        return out + [1.0 / 3.0 + 0.005 * r.uniform(-1, 1, shp)] if thermal else out
+    return fields
+
+
+def timed_step(g):
+    """One step under per-launch timing: {kind: (launches, nodes)}."""
+    g.timing(True)
+    g.step(1)
+    out = {}
+    for r in g.timing_report():
+        n, m = out.get(r["kind"], (0, 0.0))
+        out[r["kind"]] = (n + r["launches"], m + r["nodes"])
+    g.timing(False)
+    return out
+
+
+@pytest.mark.parametrize("storage", ["fp32", "fp16s", "bf16s"])
+@pytest.mark.parametrize("n,node_by_node", [
+    ((24, 24, 24), True), ((25, 9, 7), True), ((119, 25, 24), True), ((200, 6, 5), True), ((128, 8, 9), True),
+    ((20, 57, 32), True),   # 1824 tiles, the limit
+    ((20, 25, 73), False),  # 1825
+    ((129, 50, 25), None),  # 2500: 16-bit rows beyond 64 nodes go to 6080
+    ((80, 76, 80), None), ((80, 11, 553), False)])  # 6080, 6083
+def test_small_one_level_grids_run_node_by_node(n, node_by_node, storage):
+    """Few tiles: node by node by default and after autotune, on the tile
+    kernels once a variant is set, with the same bits (periodic, with walls and
+    a force)."""
+    import torch
+    if node_by_node is None:
+        node_by_node = storage != "fp32"
+    for walls, acc in (((0,) * 6, (0, 0, 0)), ((0, 0, 1, 1, 0, 0), (1e-5, 0, 0)), ((0, 0, 0, 0, 1, 1), (0, 0, 2e-5))):
+        if walls != (0,) * 6 and n[1] * n[2] > 2000:
+            continue
+        case = box(n, walls, acc)
+        a, _ = twin(case, storage, noisy(3), oracle=False)
+        b, _ = twin(case, storage, noisy(3), oracle=False)
+        a.step(2)
+        b.set_variant(1)
+        b.step(2)
+        ta, tb = timed_step(a), timed_step(b)
+        assert ("stream_collide_tma" in ta) != node_by_node and "stream_collide_tma" in tb, (ta, tb)
+        assert sum(m for _, m in ta.values()) == sum(m for _, m in tb.values()) == n[0] * n[1] * n[2]
+        assert torch.equal(a.get_populations(0), b.get_populations(0))
+    a.autotune(trials=1)
+    assert ("stream_collide_tma" in timed_step(a)) != node_by_node
