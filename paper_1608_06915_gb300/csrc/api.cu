@@ -295,7 +295,7 @@ lbm_status run_instant(lbm_grid* g, int k) {
   // TMA pass and run beside it, the explode after the pass finding them done.
   // That pays where the pass leaves the GPU idle (small grids) and costs where
   // the pass fills it, so it is a schedule variant that lbm_autotune times.
-  const bool presample = side && !hg.thermal && g->presample;
+  const bool presample = side && !hg.thermal && L > 1 && g->presample;  // one level: no samples
   if (presample) {
     cudaError_t e = cudaEventRecord(g->fwd_pre, g->stream);
     for (int q = 1; q < 3 && !e; ++q) e = cudaStreamWaitEvent(g->fwd_side[q], g->fwd_pre, 0);
