@@ -598,23 +598,35 @@ bool small_grid(const lbm_grid* g) {
 // sphere.  The 64-node tiles take over where they leave a quarter of the lanes
 // fewer idle: 27 x 53 x 108 BF16 box 0.067 ms against 0.079; at equal lanes
 // they lose (the channel 3.89 against 3.23, at 101 x 49 x 75 0.921 against
-// 0.914).  The samples run beside the pass below a
-// million node updates an instant, where the pass leaves the GPU idle (64^3
-// two-level box, 0.39 M: 0.086 ms against 0.093; reduced curved sphere, 0.5 M:
-// 0.447 against 0.461); the sphere at 4.3 M loses 6% by it.  The thermal model
-// keeps its kernel 0; FP64 patches without tiles run none of these kernels.
+// 0.914).  At FP64 kernel 1 has one stage and 3 CTAs per SM, and what counts is
+// how evenly the CTAs share the warps with nodes: the 64-node tiles also where
+// they are full (rows of a multiple of 64 nodes: 128^3 1.994 ms against 2.022,
+// 256 x 48 x 48 0.573 against 0.586, two-level 128^3 6.01 against 6.06,
+// channels of 256, 128 and 64 x 40 x 32 21.97, 11.09 and 5.69 against 22.16,
+// 11.24 and 5.77, kernel 0 there 21.86, 11.06 and 5.72; behind on 128 x 64 x
+// 64, 0.520 against 0.513, and the 128 x 32 x 32 sphere, 4.52 against 4.49),
+// but not on rows of 96, whose second half has one warp of two (96 x 64 x 64:
+// 0.521 against kernel 1's 0.402).
+// The samples run beside the pass below a million node updates an instant,
+// where the pass leaves the GPU idle (64^3 two-level box, 0.39 M: 0.086 ms
+// against 0.093; reduced curved sphere, 0.5 M: 0.447 against 0.461; FP64 48^3
+// two-level box 0.402 against 0.425); the sphere at 4.3 M loses 6% by it.  The
+// thermal model keeps its kernel 0; FP64 patches without tiles run none of
+// these kernels.
 void default_variant(lbm_grid* g) {
   if (g->hg.thermal) return;
-  double l128 = 0, l64 = 0, updates = 0;
+  double l128 = 0, l64 = 0, nodes = 0, updates = 0;
   for (const auto& p : g->hg.P) {
     const double n = (double)(1LL << p.level);
     for (int k = 0; k < 2; ++k) {
       l128 += n * 128.0 * (double)p.tiles_pure[k].size();
       l64 += n * 64.0 * (double)p.tiles_half[k].size();
+      nodes += n * p.n_tma[k];
     }
     updates += n * (double)p.n_fluid;
   }
-  g->variant = l64 <= 0.75 * l128 ? lbmk::sc_tma_variants(g->hg.desc.storage) - 1 : 1;
+  const bool full = g->hg.pop_bytes == 8 && l64 <= 1.1 * nodes;
+  g->variant = full || l64 <= 0.75 * l128 ? lbmk::sc_tma_variants(g->hg.desc.storage) - 1 : 1;
   g->presample = updates < 1e6 * (double)(1LL << (g->hg.nlev - 1));
   g->node_pass = small_grid(g);
 }
