@@ -216,7 +216,8 @@ lbm_status lbm_step(lbm_grid_t g, int64_t n_coarse_steps);
  * identical results.
  * Thermal model: 2 variants of its TMA pass (f and g stored from registers
  * straight to memory, or through a shared-memory stage by TMA), identical
- * results.  This times `trials` coarse steps of each variant
+ * results (FP64 storage has no thermal TMA pass: both run node by node).
+ * This times `trials` coarse steps of each variant
  * the way lbm_step runs them (graph replays unless lbm_graphs is off), CUDA
  * events around them, then the two fastest again over 3 * trials steps each,
  * and keeps the faster of those.  The state advances by

@@ -35,7 +35,7 @@ struct ThermalLevel {
 cudaError_t launch_th_tiles(int storage, const PatchDev& p, const void* fin, const void* gin, void* fout, void* gout,
                             const uint32_t* tiles, int64_t ntiles, int ntx, const ThermalLevel& L, int odd,
                             int* status, cudaStream_t st);
-// Thermal TMA tile pass of one patch; maps = {f load, f store, f wrap, g load,
+// Thermal TMA tile pass of one FP32 patch; maps = {f load, f store, f wrap, g load,
 // g store, g wrap} descriptors (thermal_tma.cu).  Variant 0 stores f and g
 // from registers directly to fout and gout (3 CTAs per SM); variant 1 stores
 // them through a shared-memory stage with TMA (2 CTAs per SM).

@@ -486,10 +486,12 @@ std::string build_layout(HostGrid& g) {
     // active lanes, so a patch whose rows leave more than a tenth of the tiles'
     // lanes idle goes node by node from a packed list (k_sc_nodes): rows of 100
     // nodes 0.412 ms a step against 0.513, while rows of 128 stay on the tiles.
-    // The thermal model always does, its FP64 tile pass keeps 4 warps per SM:
-    // 40 x 24 x 32 cell 4.67 ms a step against 6.96.
-    bool dense = false;
-    if (g.pop_bytes == 8) {
+    // The thermal model always does: both sets of a tile fill the shared memory
+    // of an SM, so a tile pass has 4 warps per SM.  Cells of 40, 64, 128 and 256
+    // x 24 x 32: 4.67, 7.23, 13.85 and 27.2 ms a step against 6.96, 7.40, 14.74
+    // and 28.3 on tiles, full rows included.
+    bool dense = g.pop_bytes == 8 && g.thermal;
+    if (g.pop_bytes == 8 && !g.thermal) {
       double nodes = 0, lanes = 0;
       for (int64_t row = 0; row < p.dim[1] * p.dim[2]; ++row)
         for (int64_t x0 = 0; x0 < p.dim[0]; x0 += 128) {
@@ -501,7 +503,7 @@ std::string build_layout(HostGrid& g) {
         }
       // (the tile pass carries an inlet node's populations along)
       const bool inlet = std::find(p.type.begin(), p.type.end(), (uint8_t)T_INLET) != p.type.end();
-      dense = !inlet && (g.thermal || nodes < 0.9 * lanes);
+      dense = !inlet && nodes < 0.9 * lanes;
     }
     std::vector<Rows> rows(p.dim[2]);
 #pragma omp parallel for schedule(dynamic, 1)

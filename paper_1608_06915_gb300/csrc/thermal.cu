@@ -232,12 +232,11 @@ cudaError_t launch_th_tiles(int storage, const PatchDev& p, const void* fin, con
                             const uint32_t* tiles, int64_t ntiles, int ntx, const ThermalLevel& L, int odd,
                             int* status, cudaStream_t st) {
   if (ntiles == 0) return cudaSuccess;
-  return th_dispatch(storage, [&](auto z) {
-    using R = decltype(z);
-    k_th_tiles<R><<<(unsigned)ntiles, 128, 0, st>>>(p, (const R*)fin, (const R*)gin, (R*)fout, (R*)gout, tiles, ntx,
-                                                    th_params<R>(L), odd, status);
-    return cudaGetLastError();
-  });
+  if (storage != LBM_FP32) return cudaErrorInvalidValue;  // FP64: launch_th_nodes
+  using R = float;
+  k_th_tiles<R><<<(unsigned)ntiles, 128, 0, st>>>(p, (const R*)fin, (const R*)gin, (R*)fout, (R*)gout, tiles, ntx,
+                                                  th_params<R>(L), odd, status);
+  return cudaGetLastError();
 }
 
 cudaError_t launch_th_coalesce(int storage, const PatchDev& child, const void* fin_c, const void* gin_c,

@@ -1,5 +1,6 @@
-// Thermal stream-collide through TMA: the tile pass of the two-population
+// Thermal stream-collide through TMA: the FP32 tile pass of the two-population
 // model, built like the isothermal one (sc_tma.cuh) with both sets staged.
+// (FP64 goes node by node from packed lists, k_th_nodes.)
 //
 // A tile is 128 nodes along x at one (y, z).  The producer thread loads, per
 // tile, 9 three-row boxes of f and 9 of g (one box per source row (c_y, c_z),
@@ -31,14 +32,14 @@ namespace lbmk {
 template <typename S, int OUT = 0>
 struct ThTmaCfg {
   using C = TmaCfg<S, 2>;
-  static constexpr int DI = sizeof(S) == 8 ? 1 : 2;                   // load stages
+  static constexpr int DI = 2;                                         // load stages
   static constexpr int HALF = 9 * C::GROUP + 18 * C::SIDE;             // f rows + wrap slots; g follows
   static constexpr int STAGE = 2 * HALF;
   static constexpr int OSTAGE = OUT ? 0 : 2 * 4 * C::OSEGB;           // [set][warp][population][32]
   static constexpr uint32_t TX = 2u * C::TX;
   static constexpr int SMEM = DI * STAGE + OSTAGE + 128;
   static constexpr int THREADS = 160;
-  static constexpr int MINB = (OUT && sizeof(S) == 4) ? 3 : 1;        // CTAs per SM the registers aim for
+  static constexpr int MINB = OUT ? 3 : 1;                            // CTAs per SM the registers aim for
 };
 
 template <typename S>
@@ -278,28 +279,26 @@ cudaError_t launch_th_tma(int storage, int variant, const void* const maps[6], c
                           void* fout, void* gout, const unsigned long long* tiles, int64_t ntiles,
                           const ThermalLevel& L, int* status, cudaStream_t st) {
   if (ntiles == 0) return cudaSuccess;
-  if (variant < 0 || variant > 1) return cudaErrorInvalidValue;
-  return th_dispatch(storage, [&](auto z) -> cudaError_t {
-    using R = decltype(z);
-    ThMaps<R> m;
-    memcpy(&m.f_in, maps[0], sizeof(CUtensorMap));
-    memcpy(&m.f_out, maps[1], sizeof(CUtensorMap));
-    memcpy(&m.f_wrap, maps[2], sizeof(CUtensorMap));
-    memcpy(&m.g_in, maps[3], sizeof(CUtensorMap));
-    memcpy(&m.g_out, maps[4], sizeof(CUtensorMap));
-    memcpy(&m.g_wrap, maps[5], sizeof(CUtensorMap));
-    auto go = [&](auto kern, auto cfg, int& blocks_per_sm, int& sms) -> cudaError_t {
-      using T = decltype(cfg);
-      if (cudaError_t e = th_tma_go<R, T>(kern, blocks_per_sm, sms)) return e;
-      const int grid = (int)std::min<int64_t>(ntiles, (int64_t)blocks_per_sm * sms);
-      kern<<<grid, T::THREADS, T::SMEM, st>>>(m, p, (const R*)fin, (R*)fout, (R*)gout, tiles, (int)ntiles,
-                                              th_params<R>(L), status);
-      return cudaGetLastError();
-    };
-    static int bps[2] = {-1, -1}, sms[2] = {0, 0};
-    if (variant == 0) return go(k_th_tma_d<R>, ThTmaCfg<R, 1>{}, bps[0], sms[0]);
-    return go(k_th_tma<R>, ThTmaCfg<R, 0>{}, bps[1], sms[1]);
-  });
+  if (variant < 0 || variant > 1 || storage != LBM_FP32) return cudaErrorInvalidValue;
+  using R = float;
+  ThMaps<R> m;
+  memcpy(&m.f_in, maps[0], sizeof(CUtensorMap));
+  memcpy(&m.f_out, maps[1], sizeof(CUtensorMap));
+  memcpy(&m.f_wrap, maps[2], sizeof(CUtensorMap));
+  memcpy(&m.g_in, maps[3], sizeof(CUtensorMap));
+  memcpy(&m.g_out, maps[4], sizeof(CUtensorMap));
+  memcpy(&m.g_wrap, maps[5], sizeof(CUtensorMap));
+  auto go = [&](auto kern, auto cfg, int& blocks_per_sm, int& sms) -> cudaError_t {
+    using T = decltype(cfg);
+    if (cudaError_t e = th_tma_go<R, T>(kern, blocks_per_sm, sms)) return e;
+    const int grid = (int)std::min<int64_t>(ntiles, (int64_t)blocks_per_sm * sms);
+    kern<<<grid, T::THREADS, T::SMEM, st>>>(m, p, (const R*)fin, (R*)fout, (R*)gout, tiles, (int)ntiles,
+                                            th_params<R>(L), status);
+    return cudaGetLastError();
+  };
+  static int bps[2] = {-1, -1}, sms[2] = {0, 0};
+  if (variant == 0) return go(k_th_tma_d<R>, ThTmaCfg<R, 1>{}, bps[0], sms[0]);
+  return go(k_th_tma<R>, ThTmaCfg<R, 0>{}, bps[1], sms[1]);
 }
 
 cudaError_t launch_th_nodes(int storage, const PatchDev& p, const void* fin, const void* gin, void* fout, void* gout,

@@ -95,3 +95,49 @@ def test_float32_moments_are_the_float64_ones_rounded_once(pr, storage):
     narrow = g.moments(0, dtype=torch.float32)
     for a, b in list(zip(wide, narrow))[:3 if pr is not None else 2]:
         assert torch.equal(a.float(), b)
+
+
+def plates(pr, n, **more):
+    return box(n, (0, 0, 0, 0, 1, 1),
+               thermal=dict(pr=pr, t0=1 / 3, glambda=1e-3, t_ref=1 / 3, dT=0.01,
+                            wall_T=(0, 0, 0, 0, 1 / 3 + 0.005, 1 / 3 - 0.005)), **more)
+
+
+@pytest.mark.parametrize("pr", [0.7, 2.0])
+@pytest.mark.parametrize("nx", [45, 64, 131])
+def test_thermal_tile_passes_refined_fp32_every_step(nx, pr):
+    """Both FP32 thermal tile passes on a three-level cell against the oracle.
+    A coarse step applies up to six collisions to a value (four fine steps,
+    coalesce, explode), each within 2e-6 of f and 5e-6 of g in FP32."""
+    boxes = [(lev, (0, 0, lo), (nx - 1, 8, hi)) for lev, lo, hi in
+             ((1, 0, 8), (1, 25, 33), (2, 0, 4), (2, 29, 33))]
+    case = plates(pr, (nx, 9, 34), boxes=boxes)
+    g0, o = twin(case, "fp32", noisy(11, True))
+    g1, _ = twin(case, "fp32", noisy(11, True), oracle=False)
+    g1.set_variant(1)
+    for s in range(1, 4):
+        o.step(1)
+        for g in (g0, g1):
+            g.step(1)
+            df, dg = pop_diff(g, o, 0), pop_diff(g, o, 1)
+            assert df < 6 * 2e-6 * s and dg < 6 * 5e-6 * s, (s, df, dg)
+
+
+@pytest.mark.parametrize("pr", [0.7, 2.0])
+def test_thermal_inflow_fp64_every_step(pr):
+    """FP64 thermal grids go node by node whole, beside an inlet and an outlet
+    too; inlet nodes keep their populations.  The inlet's temperature is not an
+    input of the model (the library takes T0, the oracle the field's), so both
+    step from the library's initial state."""
+    case = plates(pr, (64, 6, 8))
+    case.update(periodic=(0, 1, 0), inflow_axis=0, u_in=(0.03, 0.0, 0.0))
+    for v in (0, 1):
+        g, o = twin(case, "fp64", noisy(13, True))
+        for which in (0, 1):
+            o.set_pop(0, g.get_populations(0, which).cpu().numpy(), which)
+        g.set_variant(v)
+        for s in range(3):
+            g.step(1)
+            o.step(1)
+            df, dg = pop_diff(g, o, 0), pop_diff(g, o, 1)
+            assert df < 1e-12 and dg < 1e-12, (s, df, dg)
