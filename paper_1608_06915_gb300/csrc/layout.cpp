@@ -553,8 +553,9 @@ std::string build_layout(HostGrid& g) {
           const uint32_t id = (uint32_t)((z * p.dim[1] + y) * p.ntx + tx);
           // the TMA path fetches the periodic wrap of x-spanning rows as aligned
           // 16-byte boxes, so rows of any length can take it (a row of one node
-          // would need both wraps at once)
-          const bool wrap_ok = !p.span[0] || p.dim[0] >= 2;
+          // would need both wraps at once); a tile entry holds the x-tile, in
+          // halves too, in 16 bits, so rows beyond 32768 tiles go node by node
+          const bool wrap_ok = (!p.span[0] || p.dim[0] >= 2) && p.ntx <= 32768;
           for (int k = 0; k < 2; ++k) {
             if (active[k] == 0) continue;
             R.all[k].push_back(id);
