@@ -141,3 +141,19 @@ def test_thermal_inflow_fp64_every_step(pr):
             o.step(1)
             df, dg = pop_diff(g, o, 0), pop_diff(g, o, 1)
             assert df < 1e-12 and dg < 1e-12, (s, df, dg)
+
+
+def test_batches_of_tile_patches_fp64():
+    """Ten level-1 boxes whose rows fill their tiles: more patches with tiles
+    than one launch of the tile pass takes (8), so each instant takes two
+    launches; populations against the oracle every step."""
+    boxes = [(1, (4 + 41 * k, 8, 8), (35 + 41 * k, 16, 16)) for k in range(10)]
+    case = box((412, 24, 24), boxes=boxes)
+    for v in (0, 1, 2):
+        g, o = twin(case, "fp64", noisy(17))
+        g.set_variant(v)
+        for _ in range(2):
+            g.step(1)
+            o.step(1)
+            assert pop_diff(g, o) < 1e-12
+        assert timed_step(g)["stream_collide_tma"][0] == 4  # two instants
