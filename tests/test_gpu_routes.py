@@ -157,3 +157,19 @@ def test_batches_of_tile_patches_fp64():
             o.step(1)
             assert pop_diff(g, o) < 1e-12
         assert timed_step(g)["stream_collide_tma"][0] == 4  # two instants
+
+
+@pytest.mark.parametrize("walls", [(0,) * 6, (0, 0, 0, 0, 1, 1)])
+@pytest.mark.parametrize("nx", [29, 30, 32, 61, 62, 64, 93, 94, 126, 128, 158, 160, 189, 254, 256])
+def test_rows_that_fill_their_lanes_run_on_the_fp64_tile_pass(nx, walls):
+    """FP64 rows with at most a tenth of the lanes idle stay on the tiles: every
+    step within 1e-12 of the oracle, for every tile kernel."""
+    for v in (0, 1, 2):
+        g, o = twin(box((nx, 5, 6), walls), "fp64", noisy(nx))
+        g.set_variant(v)
+        for _ in range(3):
+            g.step(1)
+            o.step(1)
+            assert pop_diff(g, o) < 1e-12, (nx, v)
+        t = timed_step(g)
+        assert t["stream_collide_tma"] == (1, nx * 5 * 6), t
