@@ -173,3 +173,26 @@ def test_rows_that_fill_their_lanes_run_on_the_fp64_tile_pass(nx, walls):
             assert pop_diff(g, o) < 1e-12, (nx, v)
         t = timed_step(g)
         assert t["stream_collide_tma"] == (1, nx * 5 * 6), t
+
+
+def test_fixup_nodes_at_a_curved_surface_fp64():
+    """A ball with its analytic surface on rows that fill the FP64 tiles: the
+    nodes beside it are fix-up nodes, few enough for the warp-per-node kernel;
+    populations and drag against the oracle every step."""
+    c, r = (30.3, 11.8, 12.1), 6.0
+    z, y, x = np.meshgrid(np.arange(24), np.arange(24), np.arange(64), indexing="ij")
+    mask = (((x - c[0]) ** 2 + (y - c[1]) ** 2 + (z - c[2]) ** 2) < r * r).astype(np.uint8)
+    case = box((64, 24, 24), accel0=(1e-5, 0, 0), solid=dict(level=0, lo=(0, 0, 0), mask=mask),
+               wall_shape=dict(kind="sphere", c=c, r=r, solid_inside=True))
+    for v in (0, 1, 2):
+        g, o = twin(case, "fp64", noisy(19))
+        g.set_variant(v)
+        for s in range(3):
+            g.step(1)
+            o.step(1)
+            d = pop_diff(g, o)
+            assert d < 1e-12, (s, d)
+            Fg, Fo = np.array(g.drag()), o.drag()
+            assert np.max(np.abs(Fg - Fo)) < 1e-12 * np.linalg.norm(Fo), (Fg, Fo)
+        t = timed_step(g)
+        assert t["stream_collide_tma"][1] > 0 and 0 < t["stream_collide"][1] < 2000, t
