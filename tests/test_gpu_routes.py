@@ -196,3 +196,25 @@ def test_fixup_nodes_at_a_curved_surface_fp64():
             assert np.max(np.abs(Fg - Fo)) < 1e-12 * np.linalg.norm(Fo), (Fg, Fo)
         t = timed_step(g)
         assert t["stream_collide_tma"][1] > 0 and 0 < t["stream_collide"][1] < 2000, t
+
+
+@pytest.mark.parametrize("storage,stored", [("fp32", "float32"), ("fp16s", "float16"), ("bf16s", "bfloat16")])
+@pytest.mark.parametrize("nx", [4, 5, 6, 7, 8, 9, 10, 11, 12, 13, 14, 15, 31, 65, 130, 149])
+def test_periodic_wrap_at_every_offset_against_the_oracle(nx, storage, stored):
+    """One step of every tile kernel from the stored state, every place of the
+    row's last node in its 16-byte box: within the FP32 collision's 2e-6 and the
+    storage's rounding of the deviation from W_i (half a unit in the last
+    place, and half the smallest FP16 step)."""
+    import torch
+    unit = torch.finfo(getattr(torch, stored)).eps / 2
+    W = np.array([np.prod([2 / 3 if c == 1 else 1 / 6 for c in (i % 3, i // 3 % 3, i // 9)]) for i in range(27)])
+    for v in range(5):
+        g, o = twin(box((nx, 5, 6)), storage, noisy(nx))
+        g.set_variant(v)
+        o.set_pop(0, g.get_populations(0).cpu().numpy())
+        g.step(1)
+        o.step(1)
+        fo = o.get_pop(0)
+        dev = np.abs(fo - W[:, None, None, None])
+        err = np.abs(g.get_populations(0).cpu().numpy() - fo)
+        assert np.all(err <= 2e-6 + unit * (dev + 2e-6) + 2.0 ** -25), (v, np.max(err))
