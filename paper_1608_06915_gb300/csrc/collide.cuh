@@ -197,11 +197,12 @@ __device__ __forceinline__ void axis_eq_v(V u, AxisV<V>& a, bool want_inverse) {
   axis_eq_r(u, vrcp(den[0]), vrcp(den[1]), a, want_inverse);
 }
 
-// The three axes of a node.  FP64 takes the six reciprocals from that of the
-// product of the denominators (each near 1 or 2): a division there costs about
-// as many operations of the slow FP64 pipe as the fifteen products that
-// replace five of them do not; the FP32 reciprocal is one instruction of
-// another pipe.
+// The three axes of a node.  FP64 takes all six reciprocals from one division,
+// that of the product of the denominators (each near 1 or 2): fifteen products
+// in place of five divisions, which take several times as many operations of
+// the slow FP64 pipe (32^3 two-level box 1.015 times as fast, Pr = 2 thermal
+// cell 1.004; errors against 64 bits unchanged).  The FP32 reciprocal is one
+// instruction of another pipe.
 template <typename V>
 __device__ __forceinline__ void axes_eq_v(V ux, V uy, V uz, AxisV<V>& ex, AxisV<V>& ey, AxisV<V>& ez,
                                           bool want_inverse) {
@@ -279,11 +280,12 @@ __host__ __device__ constexpr int shear_class() {
 // 1/6 at +-1 and 4/6 at 0, so with the 1/6 of every axis in the tables only a
 // factor 4 is left at c = 0: a column (c_x, c_y) costs one multiply, one or
 // two FMAs and an FMA per layer, against a table of q_xy and three operations
-// a population.  The collision is bound by instruction issue (70% of the slots
-// at FP32, more with 16-bit storage) and at FP64 by the FP64 pipe, so its
-// operation count is its time: k_sc_tma's operations on a node fell by about
-// 100 of 640 (32^3 two-level box at FP64: 4.78 to 4.50 ms per ten steps; the
-// channel at FP32: 3.44 to 3.37 ms a step).
+// a population.  The collision is bound by instruction issue (with it 66% of
+// the slots at FP32, 70% before, more with 16-bit storage) and at FP64 by the
+// FP64 pipe, so its operation count is its time: the FP32 tile pass executes
+// 27.4 warp instructions per node instead of 30.1 (the channel 3.44 to 3.37 ms
+// a step), and kernel 0 takes 21.9 ms instead of 25.8 on an FP64 channel of
+// 256 x 40 x 32 (with the one division of axes_eq_v).
 template <typename V>
 struct EqTables {
   V ax[3], bx[3], bx4[3];  // per c_x: A and B of the axis, each with W1(c_x)/36; 4 B

@@ -235,8 +235,10 @@ __device__ __forceinline__ constexpr int row_base(int i) {
 // Periodic x: the first tile of a row needs, for the 9 populations with
 // c_x = +1 (i = 3j + 2), the element at x = dim - 1; the last tile, for the 9
 // with c_x = -1 (i = 3j), the element at x = 0.  Both come as 16-byte boxes
-// (map_wrap) into side slots after the 27 rows of the stage: slot j holds
-// [dim - H, dim) of population 3j + 2, slot 9 + j holds [0, H) of population 3j.
+// (map_wrap) into side slots after the 27 rows of the stage: slot j holds, of
+// population 3j + 2, the aligned box of H elements around x = dim - 1, whose
+// value is its element (dim - 1) mod H (elements beyond the row are filled with
+// zeros); slot 9 + j holds [0, H) of population 3j.
 // Every TMA destination in shared memory starts on a 128-byte boundary.
 //
 // Batching: one launch sweeps the TMA tiles of every patch stepped at an
